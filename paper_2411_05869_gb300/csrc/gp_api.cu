@@ -379,6 +379,9 @@ gp_status assemble_common(gp_ctx* ctx, const double* d_X, int64_t n, int d, cons
     dp.loff32 = upload(ctx, ps->bufs, sp.sn_loff32);
     dp.lo_off = upload(ctx, ps->bufs, sp.sn_lo_off);
     dp.doff = upload(ctx, ps->bufs, sp.sn_doff);
+    dp.op64_off = upload(ctx, ps->bufs, sp.sn_op64_off);
+    dp.upd64_fronts = upload(ctx, ps->bufs, sp.upd64_fronts);
+    dp.upd64_pre = upload(ctx, ps->bufs, sp.upd64_pre);
     dp.large_kb = upload(ctx, ps->bufs, sp.large_kb);
     dp.sn_fl = upload(ctx, ps->bufs, sp.sn_fl);
     dp.flow_fwd = upload(ctx, ps->bufs, sp.flow_fwd);
@@ -586,6 +589,9 @@ extern "C" gp_status gp_factor_core(gp_ctx* ctx, gp_pointset* ps, const gp_hyper
     if (prec == GP_FP64) {
       f->panels = dalloc<double>(ctx, f->bufs, (size_t)B * sp.panel_entries);
       f->upd = dalloc<double>(ctx, f->bufs, (size_t)B * sp.update_entries);
+      f->op64 = dalloc<__half>(ctx, f->bufs, (size_t)B * sp.op64_entries);
+      f->rho = dalloc<int32_t>(ctx, f->bufs, (size_t)B * ps->n);
+      build_digit_maps(ctx, f);
     } else {
       if (!ps->dest32) {   // the point set's own context owns (and stream-orders) its per-precision map
         compute_dest_map_mixed(ps->ctx, ps);
@@ -644,17 +650,19 @@ size_t factor_bytes(const gp_pointset* ps, gp_precision prec, int B, const Theta
   const size_t b = (size_t)B, n = (size_t)ps->n;
   size_t t = alloc_bytes((size_t)theta_stride_of(td) * b * 8) + alloc_bytes((b * n * td.n1 + 1) * 8);
   if (ps->support == 1) t += alloc_bytes(b * n * 2 * 8);   // the non-compact core's per-point sigma, Sigma
+  std::vector<char> seen(sp.sn_w.size(), 0);
+  size_t nmaps = 0;   // large fronts, each with its tensor maps
+  for (int32_t s : sp.large_fronts)
+    if (!seen[s]) {
+      seen[s] = 1;
+      nmaps++;
+    }
+  nmaps = std::max<size_t>(nmaps, 1);
   if (prec == GP_FP64) {
-    t += alloc_bytes(b * sp.panel_entries * 8) + alloc_bytes(b * sp.update_entries * 8);
+    t += alloc_bytes(b * sp.panel_entries * 8) + alloc_bytes(b * sp.update_entries * 8) +
+         alloc_bytes(b * sp.op64_entries * 2) + alloc_bytes(b * n * 4) + alloc_bytes(nmaps * 128) +
+         alloc_bytes((sp.sn_w.size() + 1) * 4);
   } else {
-    std::vector<char> seen(sp.sn_w.size(), 0);
-    size_t nmaps = 0;
-    for (int32_t s : sp.large_fronts)
-      if (!seen[s]) {
-        seen[s] = 1;
-        nmaps++;
-      }
-    nmaps = std::max<size_t>(nmaps, 1);
     t += alloc_bytes(b * sp.panel32_entries * 4) + alloc_bytes(b * sp.diag_entries * 8) +
          alloc_bytes(b * sp.update_entries * 4) + alloc_bytes(b * n * 2 * 8) + alloc_bytes(4) +
          alloc_bytes(8) +

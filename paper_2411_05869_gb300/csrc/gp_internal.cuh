@@ -10,9 +10,13 @@
 //   A8-A11 solves           solve.cu     (forward/backward supernodal solves, log-det, refinement)
 //   A12 predictive mean     predict.cu
 #pragma once
+#include <algorithm>
 #include <atomic>
 #include <mutex>
 
+#include <cuda.h>
+#include <cudaTypedefs.h>
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -162,6 +166,7 @@ void d2h(gp_ctx* ctx, T* dst, const T* src, size_t count) {
 // ------------------------------------------------------------------------------------------ symbolic plan
 // Host-side result of A6, plus the device copies the numeric kernels read.
 #define GP_GROUP 8   // default 64-column blocks per deferred-update group of the mixed path
+#define GP_GROUP64 4 // 64-column blocks per deferred-update group of the FP64 path (K = 256: f64_digits.cuh)
 #define GP_TN_LEFT 64     // tensor-core tile width (columns) of the mixed path's left-looking block updates
 #define GP_TN_GROUP 256   // default tile width of its group-end updates (rows stay 128 per tile)
 
@@ -207,9 +212,21 @@ struct SymPlan {
   std::vector<int32_t> upd_fronts;   // per step: fronts of the left-looking and of the group update
   std::vector<int64_t> upd_pre;      // their tile prefixes
 
+  // FP64 path: the digit planes of a level's large fronts (f64_digits.cuh), per front 6 planes of m rows x op64_ldk
+  // FP16 (the columns of its current group of GP_GROUP64 blocks), at sn_op64_off in a workspace of op64_entries FP16
+  // that every level and every group reuse
+  std::vector<int64_t> sn_op64_off;
+  int64_t op64_entries = 64;
+  int64_t op64_ldk(int64_t s) const {
+    return GP_TILE * std::min<int64_t>(GP_GROUP64, (sn_w[s] + GP_TILE - 1) / GP_TILE);
+  }
+  std::vector<int32_t> upd64_fronts;   // its update schedule: per launch the fronts and their tile prefix
+  std::vector<int64_t> upd64_pre;
+  struct Upd64 { int64_t off = 0, pre_off = 0, total = 0; int32_t n = 0; double flops = 0.0; };
+
   // schedule for the numeric factorization, per level
   struct EaLaunch { int64_t tab_off; int64_t ncta; };            // extend-add: CTAs of one child slot
-  struct StepLaunch { int64_t fr_off; int32_t nfront; int32_t kb; int64_t trsm_total; int64_t upd_total; int64_t pre_off;
+  struct StepLaunch { int64_t fr_off; int32_t nfront; int32_t kb; int64_t trsm_total; int64_t trsm128_total; int64_t pre_off;
                       // forward solve, steps taken in pairs (set on the first step of a pair): the tile prefix
                       // over this step's fronts, its total, and how many of them also have block kb + 1
                       int64_t pair_pre_off, pair_total; int32_t pair_n2;
@@ -224,7 +241,8 @@ struct SymPlan {
                       int64_t group_off, group_pre_off, group_total; int32_t n_group;
                       double left_flops, group_flops;
                       double left2_flops;   // the left update of block columns kb and kb + 1 together
-                      double potrf_flops, trsm_flops, upd_flops; };   // useful flops of the step's launches
+                      Upd64 left64, group64;   // the same updates of the FP64 path (128 x 64 tiles)
+                      double potrf_flops, trsm_flops; };   // useful flops of the step's launches
   struct Level {
     std::vector<EaLaunch> ea;        // one per child slot
     std::vector<EaLaunch> ea32;      // the same in chunks of GP_EA_CHUNK update-matrix entries (mixed path)
@@ -243,7 +261,7 @@ struct SymPlan {
   std::vector<int32_t> large_kb;     // block-column index of each large_fronts entry (its step)
   struct LevelLarge { int64_t off = 0; int64_t count = 0; };    // all steps' entries of a level, contiguous
   std::vector<LevelLarge> level_large;
-  std::vector<int64_t> step_pre;     // per step: prefix of TRSM tasks then of UPDATE tasks (2*(nfront+1))
+  std::vector<int64_t> step_pre;     // per step: prefix of 64-row, then of 128-row TRSM tiles (2*(nfront+1))
   std::vector<int64_t> pair_pre;     // per step pair: prefix of the paired forward-solve row tiles
   // Solves of the large fronts as one launch per level (tasks that wait for the blocks they need), with SB =
   // the level's flow_sb blocks per chain task and nbs = ceil(nb / SB) chain tasks per front:
@@ -278,6 +296,9 @@ struct DevPlan {
   int32_t* ldw;
   int64_t *loff32, *doff;
   int64_t* lo_off;
+  int64_t* op64_off;
+  int32_t* upd64_fronts;
+  int64_t* upd64_pre;
   int32_t* large_kb;
   int32_t* upd_fronts;
   int64_t* upd_pre;
@@ -342,11 +363,12 @@ struct gp_factor_s {
   float* op_lo = nullptr;       // GP_MIXED: tensor-core operands of the factored panel entries of one level's
                                 //   large fronts, B x lo_entries: the low TF32 parts (the high parts are
                                 //   panels32 itself) or, with op_f16, the FP16 pairs
-  uint8_t* op_maps = nullptr;   // GP_MIXED: TMA maps of the high and low operands, 2 x 128 bytes per updated front
+  uint8_t* op_maps = nullptr;   // TMA maps of the tensor-core operands per large front: the high and the low ones
+                                //   (GP_MIXED, 2 x 128 bytes), the digit planes (GP_FP64, 128 bytes)
   bool op_f16 = false;          // GP_MIXED: FP16 operand pairs (GP_OPT_SPLIT_F16) instead of TF32 pairs
   unsigned long long* op_dmax = nullptr;   // GP_MIXED: per proposal, the bits of max_i C_ii (FP64, >= 0): the
                                 //   FP16 pairs' power-of-two scale
-  int32_t* op_slot = nullptr;   // GP_MIXED: per supernode, its map pair (-1 = none)
+  int32_t* op_slot = nullptr;   // per supernode, its map or map pair (-1 = none)
   double* diag = nullptr;       // GP_MIXED: FP64 64 x 64 diagonal tiles, B x diag_entries
   double* delta = nullptr;      // GP_MIXED: refinement vectors (residual and correction), B x 2n
   double* dinv = nullptr;       // FP64 inverses of the 64 x 64 diagonal blocks (row-major), B x diag_entries
@@ -369,6 +391,8 @@ struct gp_factor_s {
   unsigned long long refine_runs_seen = 0;     // corrections already added to the context's launch count
   int32_t* tiles_err = nullptr; // set when a bounded wait (tensor-core updates, solve tasks) ran out
   int32_t* flow_sync = nullptr; // the solve tasks' tickets and readiness flags (flow_sync_entries)
+  __half* op64 = nullptr;       // GP_FP64: the digit planes of one level's large fronts, B x op64_entries
+  int32_t* rho = nullptr;       // GP_FP64: the scale exponent of every row of L, B x n
   double* upd = nullptr;        // B x update_entries
   float* upd32 = nullptr;
   double* val = nullptr;        // B x nnz CSR values of C_z (refinement SpMV)
@@ -431,6 +455,8 @@ void iterative_run(gp_ctx* ctx, gp_factor_t* f, int b, const double* d_resid, co
 void compute_dest_map(gp_ctx* ctx, gp_pointset* ps);
 void compute_dest_map_mixed(gp_ctx* ctx, gp_pointset* ps);
 void build_update_maps(gp_ctx* ctx, gp_factor_t* f);
+void build_digit_maps(gp_ctx* ctx, gp_factor_t* f);
+PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 int64_t bwd_part_entries(const SymPlan& sp);
 // The solve tasks' tickets (forward and backward, one each per level) and readiness flags (forward and
 // backward, B x n_fl each).

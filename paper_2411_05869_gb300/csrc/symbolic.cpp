@@ -399,6 +399,8 @@ void build_symbolic(int64_t n, const int64_t* rowptr, const int32_t* col, const 
   // ---- launch schedule
   sp.levels.assign(sp.nlevels, SymPlan::Level());
   sp.sn_lo_off.assign(sp.ns, 0);
+  sp.sn_op64_off.assign(sp.ns, 0);
+  sp.op64_entries = 64;
   sp.lo_entries = 8;
   sp.level_large.assign(sp.nlevels, SymPlan::LevelLarge());
   sp.sn_fl.assign(sp.ns, -1);
@@ -487,12 +489,36 @@ void build_symbolic(int64_t n, const int64_t* rowptr, const int32_t* col, const 
           int32_t s = sp.large_fronts[stp.fr_off + t];
           int64_t m = sp.sn_w[s] + sp.sn_r[s];
           int64_t c1 = std::min<int64_t>((int64_t)(kb + 1) * GP_TILE, sp.sn_w[s]);
-          int64_t ntr = (m - c1 + GP_TILE - 1) / GP_TILE;
-          acc += tri(ntr);
+          acc += (m - c1 + 127) / 128;
           sp.step_pre.push_back(acc);
         }
-        stp.upd_total = acc;
-        stp.potrf_flops = stp.trsm_flops = stp.upd_flops = 0.0;
+        stp.trsm128_total = acc;
+        // the FP64 path's updates: block column kb from its group's earlier blocks, and the rows and columns after
+        // the group at its last block (128 x 64 tiles)
+        auto plan64 = [&](SymPlan::Upd64& u, bool group) {
+          u.off = (int64_t)sp.upd64_fronts.size();
+          u.pre_off = (int64_t)sp.upd64_pre.size();
+          sp.upd64_pre.push_back(0);
+          for (int32_t t = 0; t < cnt; t++) {
+            const int32_t s = sp.large_fronts[stp.fr_off + t];
+            const int64_t w = sp.sn_w[s], m = w + sp.sn_r[s];
+            const int64_t c0 = (int64_t)kb * GP_TILE, c1 = std::min<int64_t>(c0 + GP_TILE, w);
+            const int64_t g0 = (int64_t)(kb / GP_GROUP64) * GP_GROUP64 * GP_TILE;
+            const int64_t gend = std::min<int64_t>(g0 + GP_GROUP64 * GP_TILE, w);
+            if (group ? (c1 < gend || gend >= m) : c0 == g0) continue;
+            sp.upd64_fronts.push_back(s);
+            const int64_t nt = (m - (group ? gend : c0) + 127) / 128;
+            u.total += group ? nt * (nt + 1) : nt;
+            sp.upd64_pre.push_back(u.total);
+            u.n++;
+            const double M = (double)(m - gend), bw = (double)(c1 - c0);
+            u.flops += group ? (double)(gend - g0) * M * (M + 1.0)
+                             : 2.0 * (double)(c0 - g0) * (bw * (bw + 1.0) / 2.0 + (double)(m - c1) * bw);
+          }
+        };
+        plan64(stp.left64, false);
+        plan64(stp.group64, true);
+        stp.potrf_flops = stp.trsm_flops = 0.0;
         for (int32_t t = 0; t < cnt; t++) {
           int32_t s = sp.large_fronts[stp.fr_off + t];
           double m = (double)sp.sn_w[s] + sp.sn_r[s];
@@ -501,7 +527,6 @@ void build_symbolic(int64_t n, const int64_t* rowptr, const int32_t* col, const 
           double M = m - c0 - bw;
           stp.potrf_flops += bw * bw * bw / 3.0;
           stp.trsm_flops += M * bw * bw;
-          stp.upd_flops += 2.0 * bw * M * (M + 1.0) / 2.0;
         }
         lv.steps.push_back(stp);
       }
@@ -537,6 +562,12 @@ void build_symbolic(int64_t n, const int64_t* rowptr, const int32_t* col, const 
         lo += (int64_t)(sp.sn_w[s] + sp.sn_r[s]) * ((sp.sn_ldw[s] + 7) / 8 * 8);
       }
       sp.lo_entries = std::max(sp.lo_entries, lo);
+      int64_t o64 = 0;   // the FP64 path's digit planes: rows of op64_ldk FP16 (a multiple of 128 bytes)
+      for (int32_t s : large) {
+        sp.sn_op64_off[s] = o64;
+        o64 += 6 * (int64_t)(sp.sn_w[s] + sp.sn_r[s]) * sp.op64_ldk(s);
+      }
+      sp.op64_entries = std::max(sp.op64_entries, o64);
     }
     // dataflow solve tasks of this level's large fronts (SB blocks of 64 columns per chain task: 2 where the
     // level's chains are long, else 1; rows below the columns in tasks of 64 SB rows): forward tasks ordered by
