@@ -28,96 +28,110 @@ __device__ __forceinline__ int rho_of(double x) {
   return e == 0 ? -1022 : e - 1022;   // |x| < 2^(e - 1022)
 }
 
-// The fixed-point form of x at scale 2^rho: round(x 2^(54 - rho)) for |x| <= 2^(rho + 1) (larger |x|, which only a failed
-// factorization has, saturate).
-__device__ __forceinline__ int64_t to_fixed(double x, int rho) {
-  const int64_t bits = __double_as_longlong(x);
-  const int e = (int)(bits >> 52) & 0x7ff;
-  const int64_t man = (bits & 0xfffffffffffffLL) | 0x10000000000000LL;
-  const int sh = 1021 + rho - e;   // right shift of the 53-bit significand
-  int64_t y;
-  if (sh <= 0) y = man << (sh < -3 ? 3 : -sh);
-  else y = sh > 54 ? 0 : (man + (1LL << (sh - 1))) >> sh;
-  if (e == 0) y = 0;
-  return bits < 0 ? -y : y;
+// A fixed-point entry is kept in units of 2^-61 of its scale 2^rho, seven bits below the last digit. Digit s > 0 plus
+// 256 is the 9-bit field at bit 7 + 9 (5 - s) of the entry plus BIAS (256 in every field, and half a digit unit, so that
+// the digits are the entry rounded); digit 0 is what is left above bit 52.
+constexpr int64_t BIAS = 64 + ((256LL << 7) | (256LL << 16) | (256LL << 25) | (256LL << 34) | (256LL << 43));
+
+// x at scale 2^rho, |x| <= 2^(rho + 1), plus BIAS (larger |x|, which only a failed factorization has, come out wrong).
+// The sign is applied as a complement: one unit of 2^-61 off for negative x.
+__device__ __forceinline__ int64_t to_biased(double x, int rho) {
+  const int hi = __double2hiint(x);
+  const uint32_t mh = (uint32_t)(hi & 0xfffff) | 0x100000u, ml = (uint32_t)__double2loint(x);
+  const int n = min(max(1024 + rho - ((hi >> 20) & 0x7ff), 0), 63);   // right shift of the significand at bit 62
+  const uint64_t man = ((uint64_t)__funnelshift_l(ml, mh, 10) << 32) | (ml << 10);
+  const int64_t sg = (int64_t)(hi >> 31);
+  return ((int64_t)(man >> n) ^ sg) + BIAS;
 }
 
-// The six digits of fixed-point y (2^-54 units): d_s + 256 sit in 9-bit fields of y plus the bias 256 (2^9 + ... +
-// 2^36 + 1); u[s] receives the field, u[0] the digit itself (taken modulo 2^12, which only a failed factorization
-// exceeds).
-__device__ __forceinline__ void digit_fields(int64_t y, uint32_t (&u)[NS]) {
-  constexpr int64_t bias = 256LL * (1 + (1LL << 9) + (1LL << 18) + (1LL << 27) + (1LL << 36));
-  const int64_t v = y + bias;
-#pragma unroll
-  for (int s = 1; s < NS; s++) u[s] = (uint32_t)((uint64_t)v >> (9 * (NS - 1 - s))) & 0x1ffu;
-  u[0] = (uint32_t)(((int32_t)(v >> 45) << 20) >> 20);
-}
-
-// Two digit fields as a pair of FP16 digits: 0x6400 + u is the FP16 number 1024 + u, and d = (1024 + u) - 1280.
-__device__ __forceinline__ uint32_t digits_half2(uint32_t ulo, uint32_t uhi) {
-  const uint32_t p = 0x64006400u + (ulo | (uhi << 16));
+// Digits s of two biased entries as a pair of FP16 numbers: 0x6400 + u is the FP16 number 1024 + u, u = d + 256.
+template <int S>
+__device__ __forceinline__ uint32_t digit_pair(int64_t va, int64_t vb) {
+  if (S == 0) {   // up to +-1024
+    uint32_t d;
+    asm("cvt.rn.f16x2.f32 %0, %1, %2;" : "=r"(d) : "f"((float)(int)(vb >> 52)), "f"((float)(int)(va >> 52)));
+    return d;
+  }
+  constexpr int SH = 7 + 9 * (NS - 1 - S);
+  const uint32_t ta = (uint32_t)((uint64_t)va >> SH);
+  const uint32_t tb = SH >= 16 ? (uint32_t)((uint64_t)vb >> (SH >= 16 ? SH - 16 : 0)) : (uint32_t)vb << (SH >= 16 ? 0 : 16 - SH);
+  const uint32_t p = ((ta & 0x1ffu) | 0x64006400u) | (tb & 0x1ff0000u);
   const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&p), __half2half2(__ushort_as_half(0x6500)));
   return *reinterpret_cast<const uint32_t*>(&d);
 }
 
-__device__ __forceinline__ uint32_t digits0_half2(uint32_t lo, uint32_t hi) {
-  const __half2 d = __halves2half2(__short2half_rn((short)lo), __short2half_rn((short)hi));
-  return *reinterpret_cast<const uint32_t*>(&d);
+// Eight consecutive entries' digits S as 16 bytes.
+template <int S>
+__device__ __forceinline__ uint4 pack8(const int64_t (&v)[8]) {
+  return make_uint4(digit_pair<S>(v[0], v[1]), digit_pair<S>(v[2], v[3]), digit_pair<S>(v[4], v[5]),
+                    digit_pair<S>(v[6], v[7]));
 }
 
-// Eight consecutive entries' digits s as 16 bytes.
-__device__ __forceinline__ uint4 pack8(const uint32_t (&u)[8][NS], int s) {
-  if (s == 0)
-    return make_uint4(digits0_half2(u[0][0], u[1][0]), digits0_half2(u[2][0], u[3][0]), digits0_half2(u[4][0], u[5][0]),
-                      digits0_half2(u[6][0], u[7][0]));
-  return make_uint4(digits_half2(u[0][s], u[1][s]), digits_half2(u[2][s], u[3][s]), digits_half2(u[4][s], u[5][s]),
-                    digits_half2(u[6][s], u[7][s]));
+// All six digits of eight consecutive entries, plane s at dst + s * plane (bytes).
+__device__ __forceinline__ void store8(uint8_t* dst, int plane, const int64_t (&v)[8]) {
+  *reinterpret_cast<uint4*>(dst) = pack8<0>(v);
+  *reinterpret_cast<uint4*>(dst + plane) = pack8<1>(v);
+  *reinterpret_cast<uint4*>(dst + 2 * plane) = pack8<2>(v);
+  *reinterpret_cast<uint4*>(dst + 3 * plane) = pack8<3>(v);
+  *reinterpret_cast<uint4*>(dst + 4 * plane) = pack8<4>(v);
+  *reinterpret_cast<uint4*>(dst + 5 * plane) = pack8<5>(v);
 }
 
-constexpr int UB = 59;   // products come out in units of 2^-59 of their scale
-
-// The levels' sums (level l weighs 2^(-18 - 9 l)) as a fixed-point number in units of 2^-q; what the caller knows to
-// be below 2^(63 - q) comes out right whatever the size of the single levels (integer arithmetic modulo 2^64).
-__device__ __forceinline__ int64_t combine_at(const float (&a)[NL], int q) {
-  int64_t t1 = (int64_t)__float2int_rn(a[0]) * (1LL << 27);
-  t1 += (int64_t)__float2int_rn(a[1]) * (1LL << 18);
-  t1 += (int64_t)__float2int_rn(a[2]) * (1LL << 9);
-  t1 += (int64_t)__float2int_rn(a[3]);                       // levels 0..3 in units of 2^-45
-  int64_t t0 = (int64_t)__float2int_rn(a[4]) * (1LL << 18);
-  t0 += (int64_t)__float2int_rn(a[5]) * (1LL << 9);
-  t0 += (int64_t)__float2int_rn(a[6]);                       // levels 4..6 in units of 2^-72
-  const int s1 = q - 45, s0 = 72 - q;
-  t1 = s1 >= 0 ? (s1 > 63 ? 0 : (int64_t)((uint64_t)t1 << s1)) : t1 >> min(63, -s1);
-  t0 = s0 > 0 ? (t0 + (1LL << min(62, s0 - 1))) >> min(63, s0) : (s0 < -63 ? 0 : (int64_t)((uint64_t)t0 << -s0));
-  return t1 + t0;
+// A number in floating form: sign, significand n (leading bit 62, or 0) and the exponent e of its value n 2^(e - 62).
+struct Norm {
+  uint64_t n;
+  int32_t sg;   // 0 or -1
+  int e;
+};
+// v 2^(e0 - 62) for |v| < 2^63.
+__device__ __forceinline__ Norm normalise(int64_t v, int e0) {
+  Norm r;
+  r.sg = (int32_t)(v >> 63);
+  const int64_t s64 = (int64_t)r.sg;
+  const uint64_t a = (uint64_t)((v ^ s64) - s64);
+  const int z = __clzll((long long)a) - 1;   // 0..62 (63 for v = 0)
+  r.n = a << z;
+  r.e = e0 - z;
+  return r;
 }
-
-// The same at q = UB for the dot product of two rows of a Cholesky factor (at most 4).
-__device__ __forceinline__ int64_t combine(const float (&a)[NL]) {
-  constexpr int S = UB - 18;   // shift of level 0
-  const float low = fmaf(a[6], 0x1p-13f, a[5] * 0x1p-4f);   // levels 5 and 6, rounded to a unit
-  int64_t v = (int64_t)__float2int_rn(a[0]) * (1LL << S);
-  v += (int64_t)__float2int_rn(a[1]) * (1LL << (S - 9));
-  v += (int64_t)__float2int_rn(a[2]) * (1LL << (S - 18));
-  v += (int64_t)__float2int_rn(a[3]) * (1LL << (S - 27));
-  v += (int64_t)__float2int_rn(a[4]) * (1LL << (S - 36));
-  return v + (int64_t)__float2int_rn(low);
+// Rounded to FP64 (half away from zero; below the normal range: 0), in integers: the FP64 pipe is the slow one here.
+__device__ __forceinline__ double to_double(const Norm& r) {
+  const uint64_t man = (r.n + 512) >> 10;   // 2^52 <= man <= 2^53
+  const int E = 1022 + r.e;                 // the biased exponent less one: man brings the other one
+  uint32_t hi = (uint32_t)(man >> 32) + ((uint32_t)min(E, 2045) << 20), lo = (uint32_t)man;
+  const bool zero = r.n == 0 || E <= 0;
+  hi = zero ? 0u : hi | ((uint32_t)r.sg & 0x80000000u);
+  lo = zero ? 0u : lo;
+  return __hiloint2double((int)hi, (int)lo);
 }
-
-// v 2^(rho - UB) rounded to FP64 (half away from zero), in integers: the FP64 pipe is the slow one here.
-__device__ __forceinline__ double to_double(int64_t v, int rho) {
-  if (v == 0) return 0.0;
-  const uint64_t a = (uint64_t)(v < 0 ? -v : v);
-  const int z = __clzll((long long)a);
-  const uint64_t nrm = a << z;
-  const uint64_t man = (nrm >> 11) + ((nrm >> 10) & 1);    // 2^52 <= man <= 2^53
-  const int E = 1023 + 62 - UB + 1 - z + rho;              // biased exponent of man / 2^52
-  if (E <= 0) return 0.0;                                  // below the normal range
-  const uint64_t bits = ((uint64_t)(E < 2046 ? E - 1 : 2045) << 52) + man;
-  return __longlong_as_double((long long)(bits | ((uint64_t)v & 0x8000000000000000ull)));
+// The same number as a biased fixed-point entry at scale 2^rho.
+__device__ __forceinline__ int64_t to_biased(const Norm& r, int rho) {
+  const int n = min(max(rho + 1 - r.e, 0), 63);
+  return ((int64_t)(r.n >> n) ^ (int64_t)r.sg) + BIAS;
 }
+__device__ __forceinline__ double fix2double(int64_t v, int e) { return to_double(normalise(v, e + 62)); }   // v 2^e
 
-// Fixed-point form in 2^-54 units (to_fixed's) of v in 2^-UB units.
-__device__ __forceinline__ int64_t refix(int64_t v) { return (v + (1LL << (UB - 55))) >> (UB - 54); }
+// The levels' sums (level l weighs 2^(-18 - 9 l) of the product of the two scales, 2^e) as one number.
+__device__ __forceinline__ int64_t high_levels(const float (&a)[NL]) {   // levels 0..3 in units of 2^-45
+  int64_t t = (int64_t)__float2int_rn(a[0]) * (1 << 27);
+  t += (int64_t)__float2int_rn(a[1]) * (1 << 18);
+  t += (int64_t)__float2int_rn(a[2]) * (1 << 9);
+  return t + (int64_t)__float2int_rn(a[3]);
+}
+// The dot product of two rows of a Cholesky factor (at most 4): units of 2^-59. Levels 4 to 6 are added in FP32 before
+// the conversion (at most 2^30 units, and the sum's rounding matters only where the diagonal's squares make it large).
+__device__ __forceinline__ Norm product_rows(const float (&a)[NL], int e) {
+  const float low = fmaf(a[6], 0x1p-13f, fmaf(a[5], 0x1p-4f, a[4] * 0x1p5f));
+  return normalise(high_levels(a) * (1LL << 14) + (int64_t)__float2int_rn(low), e + 3);
+}
+// A dot product of 64 terms of at most 1 that the caller knows to be at most 2^eb: units of 2^(eb - 61) where the levels
+// give that much, 2^-55 of the scales at the coarsest (the 64 terms' bound), 2^-69 at the finest.
+__device__ __forceinline__ Norm product_any(const float (&a)[NL], int e, int eb) {
+  const int S = 16 - max(min(eb - e, 6), -8);   // extra bits below the levels 0..3
+  const float low = fmaf(a[6], 0x1p-27f, a[5] * 0x1p-18f) * __int_as_float((127 + S) << 23);
+  int64_t v = high_levels(a) << S;
+  v += (int64_t)__float2int_rn(a[4]) * (int64_t)(1 << (S - 9));
+  return normalise(v + (int64_t)__float2int_rn(low), e + 17 - S);
+}
 
 }  // namespace f64d

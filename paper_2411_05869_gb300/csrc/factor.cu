@@ -25,7 +25,7 @@
 
 #include "f64_digits.cuh"
 #include "gp_internal.cuh"
-#include "potrf_tile.cuh"
+#include "potrf64.cuh"
 #include "tc_gemm.cuh"
 
 void values_run(gp_ctx* ctx, gp_factor_t* f);
@@ -141,20 +141,29 @@ __device__ __forceinline__ int find_front(const int64_t* pre, int nfront, int64_
   return lo;
 }
 
-// POTRF of the diagonal tile of block column kb and its inverse (row-major, for the TRSM and the solves), one CTA per
-// large front.
-__global__ void __launch_bounds__(POTRF_THREADS) k_potrf64(const int32_t* __restrict__ fronts, int kb, DevPlan dp,
-                                                           double* __restrict__ panels, int64_t PE,
-                                                           int32_t* __restrict__ notpd, double* __restrict__ dinv,
-                                                           int64_t DE) {
-  const int32_t s = fronts[blockIdx.x];
+// POTRF of the diagonal tile of block column kb, its inverse in FP64 (row-major, for the solves) and the inverse's digit
+// planes for the step's TRSM, a cluster of two CTAs per large front.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(p64::THREADS, 1)
+    k_potrf64(const int32_t* __restrict__ fronts, int kb, DevPlan dp, double* __restrict__ panels, int64_t PE,
+              int32_t* __restrict__ notpd, double* __restrict__ dinv, int64_t DE, uint8_t* __restrict__ itile,
+              int64_t IE, int32_t* __restrict__ err) {
+  extern __shared__ __align__(16) uint8_t potrf_raw[];
+  p64::Smem& sm = *reinterpret_cast<p64::Smem*>(potrf_raw);
+  const int fi = blockIdx.x >> 1;
+  const int32_t s = fronts[fi];
   const int b = blockIdx.y;
   const int w = dp.w[s];
   const int64_t m = (int64_t)w + dp.r[s];
-  const int c0 = kb * T;
-  potrf_tile<double, double, true, true>(panels + (int64_t)b * PE + dp.loff[s] + (int64_t)c0 * m + c0, 1, m,
-                                         dinv + (int64_t)b * DE + dp.doff[s] + (int64_t)kb * T * T, min(T, w - c0),
-                                         dp.sn_first[s] + c0, notpd + b);
+  const int c0 = kb * T, bw = min(T, w - c0);
+  const int32_t first = dp.sn_first[s] + c0;
+  double* P = panels + (int64_t)b * PE + dp.loff[s] + (int64_t)c0 * m + c0;
+  if (threadIdx.x < 3 * T) tcg::mbar_init(&sm.lready[threadIdx.x], 1);   // the three arrays
+  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  tcg::cluster_sync();
+  if (tcg::cluster_ctarank() == 0) p64::factor(sm, P, m, bw, first, notpd + b, err);
+  else p64::inverse(sm, dinv + (int64_t)b * DE + dp.doff[s] + (int64_t)kb * T * T,
+                    itile + (int64_t)b * IE + (int64_t)fi * p64::TILE_BYTES, bw, err);
+  tcg::cluster_sync();   // no CTA leaves while the other may write into it
 }
 
 // rho of every row of L (permuted order): sqrt(C_jj) <= 2^(rho + 1), from the exponent of the assembled diagonal; |L_ji| <= sqrt(C_jj) makes it a scale for the digits of the whole row.
@@ -203,91 +212,80 @@ __device__ __forceinline__ void tmem_ld_levels(uint32_t ta, int ld, float (&a)[f
 }
 
 // TRSM of the rows below diagonal tile kb as X = B inv(L_11)^T on the tensor cores: one CTA of 256 threads per 128-row
-// tile, thread (row, half) holding 32 of the row's 64 entries. The rows of B and of the inverse are cut into digits
-// at the exponent of their largest entry, straight into 128-byte-swizzled operand tiles; 26 digit products of 128 x
-// 64 x 64 follow, one TMEM accumulator per level; each thread then rounds its row's entries of X to FP64 for the
-// panel and cuts them into the digits the updates read (at the row's scale rho). Bounded by latency at the top levels
-// (one wave of CTAs: load, cut, multiply, store in turn): 38 us per launch at n = 100k, 117 us as an FP64
-// substitution column by column.
+// tile, thread (row, half) holding 32 of the row's 64 entries. The rows of B (times the 2^-sigma of the inverse's columns)
+// are cut into digits at the exponent of their largest entry, straight into 128-byte-swizzled operand tiles, while the
+// inverse's planes arrive by one bulk copy; 26 digit products of 128 x 64 x 64 follow, one TMEM accumulator per level;
+// each thread then rounds its row's entries of X to FP64 for the panel and cuts them into the digits the updates read (at
+// the row's scale rho), which leave through shared memory by TMA (a thread's own 16-byte stores would touch one line
+// each). Bounded by latency at the top levels (one wave of CTAs: load, cut, multiply, store in turn): 21 us a launch with
+// one tile, 117 us as an FP64 substitution column by column.
 constexpr int TRSM_ROWS = 128;
-constexpr int TRSM_PLANE_A = TRSM_ROWS * 128, TRSM_PLANE_B = T * 128;   // bytes of one digit plane
-constexpr int TRSM_SMEM = f64d::NS * (TRSM_PLANE_A + TRSM_PLANE_B) + 1024;
+constexpr int TRSM_PLANE_A = TRSM_ROWS * 128;   // bytes of one digit plane of B
+constexpr int TRSM_SMEM = f64d::NS * TRSM_PLANE_A + p64::TILE_BYTES + 1024;
 
 __global__ void __launch_bounds__(256, 1)
     k_trsm64(const int32_t* __restrict__ fronts, const int64_t* __restrict__ pre, int nfront, int kb, DevPlan dp,
-             double* __restrict__ panels, int64_t PE, const double* __restrict__ dinv, int64_t DE,
-             const int32_t* __restrict__ rho, int64_t n, __half* __restrict__ ops, int64_t OE,
-             int32_t* __restrict__ err, tcg::WaitLimit lim) {
+             double* __restrict__ panels, int64_t PE, const uint8_t* __restrict__ itile, int64_t IE,
+             const int32_t* __restrict__ rho, int64_t n, const uint8_t* __restrict__ tmaps,
+             const int32_t* __restrict__ slot_of, int32_t* __restrict__ err, tcg::WaitLimit lim) {
   using namespace f64d;
   extern __shared__ __align__(1024) uint8_t trsm_raw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)trsm_raw + 1023) & ~(uintptr_t)1023);
-  __shared__ uint64_t bar;
+  uint8_t* inv = sm + NS * TRSM_PLANE_A;
+  const int32_t* einv = reinterpret_cast<const int32_t*>(inv + NS * p64::PLANE);   // rows' exponents, columns' sigma
+  __shared__ uint64_t bar, ibar;
   __shared__ uint32_t tslot;
-  __shared__ int emax_s[2][TRSM_ROWS], rinv_s[T], skip_s;
+  __shared__ int emax_s[2][TRSM_ROWS], skip_s;
   const int tid = threadIdx.x, warp = tid >> 5;
   const int row = tid & 127, half = tid >> 7;
-  if (tid == 0) {
-    tcg::mbar_init(&bar, 1);
-    skip_s = *(volatile int32_t*)err;   // an earlier launch of this factorization ran out of a wait
-    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
-  }
-  if (warp == 0) tcg::tmem_alloc(&tslot, 512);
   const int64_t t = blockIdx.x;
   const int fi = find_front(pre, nfront, t);
-  const int32_t s = fronts[fi];
   const int b = blockIdx.y;
+  if (tid == 0) {
+    tcg::mbar_init(&bar, 1);
+    tcg::mbar_init(&ibar, 1);
+    skip_s = *(volatile int32_t*)err;   // an earlier launch of this factorization ran out of a wait
+    asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+    tcg::mbar_arrive_expect_tx(&ibar, p64::TILE_BYTES);
+    tcg::bulk_load(tcg::smem_u32(inv), itile + (int64_t)b * IE + (int64_t)fi * p64::TILE_BYTES, p64::TILE_BYTES, &ibar);
+  }
+  if (warp == 0) tcg::tmem_alloc(&tslot, 512);
+  const int32_t s = fronts[fi];
   const int w = dp.w[s], r = dp.r[s];
   const int64_t m = (int64_t)w + r;
   const int c0 = kb * T, bw = min(T, w - c0), c1 = c0 + bw;
   const int64_t r0 = c1 + (t - pre[fi]) * TRSM_ROWS;
   const int nr = (int)imin64(TRSM_ROWS, m - r0);
-  double* P = panels + (int64_t)b * PE + dp.loff[s] + (int64_t)c0 * m + r0;
   const bool rok = row < nr;
+  double* P = panels + (int64_t)b * PE + dp.loff[s] + (int64_t)(c0 + 32 * half) * m + r0 + row;   // this thread's entries
+  const int nc = min(max(bw - 32 * half, 0), rok ? 32 : 0);
+  const int32_t rr = rok ? rho[(int64_t)b * n + dp.frows[dp.frow_off[s] + r0 + row]] : 0;
+  int rx;
   {
     double x[32];
+    const double* p = P;
 #pragma unroll
-    for (int c = 0; c < 32; c++) x[c] = rok && 32 * half + c < bw ? P[(32 * half + c) * m + row] : 0.0;
-    // the inverse: thread (q, quarter), 16 entries of row q
-    const int q = tid >> 2, l0 = (tid & 3) * 16;
-    const double2* iv = reinterpret_cast<const double2*>(dinv + (int64_t)b * DE + dp.doff[s] + (int64_t)kb * T * T + q * T + l0);
-    double y[16];
-#pragma unroll
-    for (int c = 0; c < 8; c++) {
-      const double2 v = iv[c];
-      y[2 * c] = v.x;
-      y[2 * c + 1] = v.y;
+    for (int c = 0; c < 32; c++, p += m) x[c] = c < nc ? *p : 0.0;
+    __syncthreads();   // ibar is initialised
+    if (!tcg::mbar_wait(&ibar, 0, lim)) {
+      atomicExch(err, 1);
+      tcg::mbar_wait(&ibar, 0);   // the copy must land before the CTA ends
     }
-    int ey = 0, ex = 0;
+    int ex = -4096;
 #pragma unroll
-    for (int c = 0; c < 16; c++) ey = max(ey, __double2hiint(y[c]) & 0x7ff00000);
-    ey = max(ey, __shfl_xor_sync(0xffffffffu, ey, 1));
-    ey = max(ey, __shfl_xor_sync(0xffffffffu, ey, 2));
-    const int ry = rho_of(__hiloint2double(ey, 0));
-    if ((tid & 3) == 0) rinv_s[q] = ry;
-#pragma unroll
-    for (int g = 0; g < 2; g++) {
-      uint32_t u[8][NS];
-#pragma unroll
-      for (int c = 0; c < 8; c++) digit_fields(to_fixed(y[8 * g + c], ry), u[c]);
-      const uint32_t o = q * 128 + ((((l0 >> 3) + g) ^ (q & 7)) << 4);
-#pragma unroll
-      for (int d = 0; d < NS; d++)
-        *reinterpret_cast<uint4*>(sm + NS * TRSM_PLANE_A + d * TRSM_PLANE_B + o) = pack8(u, d);
+    for (int c = 0; c < 32; c++) {
+      const int e = (__double2hiint(x[c]) >> 20) & 0x7ff;
+      ex = max(ex, e == 0 ? -4096 : e - einv[T + 32 * half + c]);
     }
-#pragma unroll
-    for (int c = 0; c < 32; c++) ex = max(ex, __double2hiint(x[c]) & 0x7ff00000);
     emax_s[half][row] = ex;
     __syncthreads();
-    ex = max(ex, emax_s[half ^ 1][row]);
-    const int rx = rho_of(__hiloint2double(ex, 0));
+    rx = max(max(ex, emax_s[half ^ 1][row]) - 1022, -900);   // |x| 2^-sigma < 2^rx
 #pragma unroll
     for (int g = 0; g < 4; g++) {
-      uint32_t u[8][NS];
+      int64_t v[8];
 #pragma unroll
-      for (int c = 0; c < 8; c++) digit_fields(to_fixed(x[8 * g + c], rx), u[c]);
-      const uint32_t o = row * 128 + (((4 * half + g) ^ (row & 7)) << 4);
-#pragma unroll
-      for (int d = 0; d < NS; d++) *reinterpret_cast<uint4*>(sm + d * TRSM_PLANE_A + o) = pack8(u, d);
+      for (int c = 0; c < 8; c++) v[c] = to_biased(x[8 * g + c], rx + einv[T + 32 * half + 8 * g + c]);
+      store8(sm + row * 128 + (((4 * half + g) ^ (row & 7)) << 4), TRSM_PLANE_A, v);
     }
   }
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");   // the operand tiles are visible to the tensor core
@@ -297,7 +295,7 @@ __global__ void __launch_bounds__(256, 1)
   const uint32_t tmem = tslot;
   const bool skip = skip_s != 0;
   if (tid == 0 && !skip) {
-    const uint32_t sa = tcg::smem_u32(sm), sb = sa + NS * TRSM_PLANE_A;
+    const uint32_t sa = tcg::smem_u32(sm), sb = tcg::smem_u32(inv);
     const uint32_t idesc = tcg::idesc_f16(TRSM_ROWS, T);
 #pragma unroll 1
     for (int l = 0; l < NL; l++)
@@ -305,7 +303,7 @@ __global__ void __launch_bounds__(256, 1)
 #pragma unroll
         for (int kk = 0; kk < 4; kk++)
           tcg::mma_f16(tmem + l * T, tcg::smem_desc_sw128(sa + d * TRSM_PLANE_A + kk * 32),
-                       tcg::smem_desc_sw128(sb + (l - d) * TRSM_PLANE_B + kk * 32), idesc,
+                       tcg::smem_desc_sw128(sb + (l - d) * p64::PLANE + kk * 32), idesc,
                        d > max(0, l - NS + 1) || kk > 0);
     tcg::mma_commit(&bar);
   }
@@ -318,34 +316,37 @@ __global__ void __launch_bounds__(256, 1)
   ok = ok && !skip;
   __syncwarp();
   tcg::tc_fence_after();
-  const int32_t rr = rok ? rho[(int64_t)b * n + dp.frows[dp.frow_off[s] + r0 + row]] : 0;
-  const int rx = rho_of(__hiloint2double(max(emax_s[0][row], emax_s[1][row]), 0));
-  const int ldk = ldk_of(w);
-  __half* H = ops + (int64_t)b * OE + dp.op64_off[s] + (r0 + row) * ldk + (kb % KB) * T + 32 * half;
-  const int64_t plane = m * ldk;
+  {
+    double* p = P;
 #pragma unroll 1
-  for (int g = 0; g < 4; g++) {
-    float a[NL][8];
-    tmem_ld_levels(tmem + ((uint32_t)((warp & 3) * 32) << 16) + 32 * half + 8 * g, T, a);
-    uint32_t u[8][NS];
+    for (int g = 0; g < 4; g++) {
+      float a[NL][8];
+      tmem_ld_levels(tmem + ((uint32_t)((warp & 3) * 32) << 16) + 32 * half + 8 * g, T, a);
+      int64_t v[8];
 #pragma unroll
-    for (int c = 0; c < 8; c++) {
-      const float al[NL] = {a[0][c], a[1][c], a[2][c], a[3][c], a[4][c], a[5][c], a[6][c]};
-      const int j = 32 * half + 8 * g + c;
-      const int64_t v = combine_at(al, UB + rx + rinv_s[j] - rr);   // X in units of 2^(rr - UB): |X| <= 2^(rr + 1)
-      if (ok && rok && j < bw) P[(int64_t)j * m + row] = to_double(v, rr);
-      digit_fields(refix(v), u[c]);
-    }
-    if (ok && rok) {
-#pragma unroll
-      for (int d = 0; d < NS; d++) *reinterpret_cast<uint4*>(H + d * plane + 8 * g) = pack8(u, d);
+      for (int c = 0; c < 8; c++, p += m) {
+        const float al[NL] = {a[0][c], a[1][c], a[2][c], a[3][c], a[4][c], a[5][c], a[6][c]};
+        const Norm x = product_any(al, rx + einv[32 * half + 8 * g + c], rr + 1);
+        if (ok && 8 * g + c < nc) *p = to_double(x);
+        v[c] = to_biased(x, rr);
+      }
+      store8(sm + row * 128 + (((4 * half + g) ^ (row & 7)) << 4), TRSM_PLANE_A, v);
     }
   }
+  asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   tcg::tc_fence_before();
   __syncthreads();
   if (warp == 0) {
     tcg::tc_fence_after();
     tcg::tmem_dealloc(tmem, 512);
+  }
+  if (tid == 0 && ok) {   // the digits of X: 64-row boxes, rows past the front are not written
+    const uint8_t* map = tmaps + (int64_t)slot_of[s] * 128;
+    tcg::tmap_acquire(map);
+    for (int h = 0; h < 2 && h * T < nr; h++)
+      for (int d = 0; d < NS; d++)
+        tcg::tma_store_4d(map, kb % KB * T, (int)r0 + h * T, d, b, tcg::smem_u32(sm) + d * TRSM_PLANE_A + h * T * 128);
+    tcg::bulk_store_wait();
   }
 }
 
@@ -360,7 +361,7 @@ __global__ void __launch_bounds__(256, 1)
 // memory, so a tile's epilogue does not overlap the next tile's MMAs (its operand loads do). 128 x 64 x 16
 // instructions read 6 KB of shared memory in the 32 clocks they multiply: about two thirds of the FP16 peak.
 // Against FP64 multiply-adds (64-column updates of the whole trailing matrix at the FP64 pipe's 1 TFLOP/s) the updates
-// of one factorization went from 101.8 to 10.6 ms at n = 100k (1.1e11 flops) and from 725 to 47 ms at n = 200k (8.3e11
+// of one factorization went from 101.8 to 9.4 ms at n = 100k (1.1e11 flops) and from 725 to 42 ms at n = 200k (8.3e11
 // flops); residuals |r - C alpha| / |r| stayed the same.
 constexpr int U64_THREADS = 320, U64_SLOTS = 9, U64_SLOT = (128 + T) * 128;
 constexpr int U64_SMEM = U64_SLOTS * U64_SLOT + 256 + 1024;
@@ -559,6 +560,9 @@ __global__ void __launch_bounds__(U64_THREADS, 1)
       }
       const int ri = i < u.m ? rb[rows[i]] : 0;
       const int rjl = jb + lane < u.jlim ? rb[rows[jb + lane]] : 0;   // lane l: column jb + l
+      const int nv = i < u.m ? (int)imin64(32, imin64(i + 1, u.jlim) - jb) : 0;   // this row's entries: the first nv columns
+      double* p = colp(jb) + i;   // dereferenced only below nv
+      int wl = (int)imin64(64, u.w - jb);   // columns from wl on lie in the update matrix
       if (!tcg::mbar_wait(tfull, aph, lim)) {
         fail();
         break;
@@ -567,12 +571,14 @@ __global__ void __launch_bounds__(U64_THREADS, 1)
       tcg::tc_fence_after();
 #pragma unroll 1
       for (int g = 0; g < 4; g++) {
-        const int64_t j0 = jb + 8 * g;
         double old[8];
+        double* pc[8];
 #pragma unroll
         for (int c = 0; c < 8; c++) {
-          const int64_t j = j0 + c;
-          old[c] = i < u.m && j <= i && j < u.jlim ? colp(j)[i] : 0.0;
+          const int j = 8 * g + c;
+          pc[c] = p;
+          old[c] = j < nv ? *p : 0.0;
+          p = j + 1 == wl ? U + (i - u.w) : p + (j < wl ? u.m : (int64_t)u.r);
         }
         float a[NL][8];
         tmem_ld_levels(tmem + ((uint32_t)(q * 32) << 16) + 32 * h + 8 * g, T, a);
@@ -583,11 +589,10 @@ __global__ void __launch_bounds__(U64_THREADS, 1)
         }
 #pragma unroll
         for (int c = 0; c < 8; c++) {
-          const int64_t j = j0 + c;
           const float al[NL] = {a[0][c], a[1][c], a[2][c], a[3][c], a[4][c], a[5][c], a[6][c]};
           const int rj = __shfl_sync(0xffffffffu, rjl, 8 * g + c);
-          const double v = to_double(combine(al), ri + rj);
-          if (i < u.m && j <= i && j < u.jlim) colp(j)[i] = old[c] - v;
+          const double v = to_double(product_rows(al, ri + rj));
+          if (8 * g + c < nv) *pc[c] = old[c] - v;
         }
       }
       aph ^= 1;
@@ -619,6 +624,7 @@ void set_attrs() {   // once per process (contexts may run on several host threa
   std::call_once(g_attrs_once, [] {
     GP_CUDA(cudaFuncSetAttribute(k_small_front, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  GP_SMALL_M * GP_SMALL_M * (int)sizeof(double)));
+    GP_CUDA(cudaFuncSetAttribute(k_potrf64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(p64::Smem)));
     GP_CUDA(cudaFuncSetAttribute(k_trsm64, cudaFuncAttributeMaxDynamicSharedMemorySize, TRSM_SMEM));
     GP_CUDA(cudaFuncSetAttribute(k_update64<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, U64_SMEM));
     GP_CUDA(cudaFuncSetAttribute(k_update64<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, U64_SMEM));
@@ -660,7 +666,7 @@ static void factor_body(gp_ctx* ctx, gp_factor_t* f) {
   cudaStream_t st = ctx->stream;
   set_attrs();
   const int B = f->B;
-  const int64_t PE = sp.panel_entries, UE = sp.update_entries;
+  const int64_t PE = sp.panel_entries, UE = sp.update_entries, IE = itile_bytes(sp);
   values_run(ctx, f);   // A3, A4 (zeroes and fills the panels)
   k_fill_i32<<<grid_for(B, 128), 128, 0, st>>>(f->notpd, B, INT_MAX);
   GP_CHECK_LAUNCH(ctx);
@@ -708,21 +714,23 @@ static void factor_body(gp_ctx* ctx, gp_factor_t* f) {
       if (stp.left64.total > 0) update(stp.left64, stp.kb, false);
       {
         ProfScope ps_(ctx, KC_POTRF, B * stp.potrf_flops);
-        k_potrf64<<<dim3(stp.nfront, B), POTRF_THREADS, 0, st>>>(fronts, stp.kb, dp, f->panels, PE, f->notpd, f->dinv,
-                                                                 sp.diag_entries);
+        k_potrf64<<<dim3(2 * stp.nfront, B), p64::THREADS, sizeof(p64::Smem), st>>>(
+            fronts, stp.kb, dp, f->panels, PE, f->notpd, f->dinv, sp.diag_entries, f->itile, IE, f->tiles_err);
         GP_CHECK_LAUNCH(ctx);
       }
       if (stp.trsm128_total > 0) {
         ProfScope ps_(ctx, KC_TRSM, B * stp.trsm_flops);
         k_trsm64<<<dim3((unsigned)stp.trsm128_total, B), 256, TRSM_SMEM, st>>>(
-            fronts, dp.step_pre + stp.pre_off + stp.nfront + 1, stp.nfront, stp.kb, dp, f->panels, PE, f->dinv,
-            sp.diag_entries, f->rho, ps->n, f->op64, sp.op64_entries, f->tiles_err, f->wait_lim);
+            fronts, dp.step_pre + stp.pre_off + stp.nfront + 1, stp.nfront, stp.kb, dp, f->panels, PE, f->itile, IE,
+            f->rho, ps->n, f->op_maps, f->op_slot, f->tiles_err, f->wait_lim);
         GP_CHECK_LAUNCH(ctx);
       }
       if (stp.group64.total > 0) update(stp.group64, stp.kb, true);
     }
   }
 }
+
+int64_t itile_bytes(const SymPlan& sp) { return sp.max_large * (int64_t)p64::TILE_BYTES; }
 
 // The tensor maps of the FP64 path's digit planes, one per large front: 4-D (columns of a group x rows x digit planes x
 // proposals), boxes of 64 columns x 64 rows with the 128-byte swizzle; rows past the front read as zeros.

@@ -590,6 +590,7 @@ extern "C" gp_status gp_factor_core(gp_ctx* ctx, gp_pointset* ps, const gp_hyper
       f->panels = dalloc<double>(ctx, f->bufs, (size_t)B * sp.panel_entries);
       f->upd = dalloc<double>(ctx, f->bufs, (size_t)B * sp.update_entries);
       f->op64 = dalloc<__half>(ctx, f->bufs, (size_t)B * sp.op64_entries);
+      f->itile = dalloc<uint8_t>(ctx, f->bufs, (size_t)B * itile_bytes(sp));
       f->rho = dalloc<int32_t>(ctx, f->bufs, (size_t)B * ps->n);
       build_digit_maps(ctx, f);
     } else {
@@ -660,7 +661,7 @@ size_t factor_bytes(const gp_pointset* ps, gp_precision prec, int B, const Theta
   nmaps = std::max<size_t>(nmaps, 1);
   if (prec == GP_FP64) {
     t += alloc_bytes(b * sp.panel_entries * 8) + alloc_bytes(b * sp.update_entries * 8) +
-         alloc_bytes(b * sp.op64_entries * 2) + alloc_bytes(b * n * 4) + alloc_bytes(nmaps * 128) +
+         alloc_bytes(b * sp.op64_entries * 2) + alloc_bytes(b * itile_bytes(sp)) + alloc_bytes(b * n * 4) + alloc_bytes(nmaps * 128) +
          alloc_bytes((sp.sn_w.size() + 1) * 4);
   } else {
     t += alloc_bytes(b * sp.panel32_entries * 4) + alloc_bytes(b * sp.diag_entries * 8) +

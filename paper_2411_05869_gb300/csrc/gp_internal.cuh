@@ -217,6 +217,7 @@ struct SymPlan {
   // that every level and every group reuse
   std::vector<int64_t> sn_op64_off;
   int64_t op64_entries = 64;
+  int64_t max_large = 1;   // most large fronts of a level (the FP64 path's inverse tiles of one step)
   int64_t op64_ldk(int64_t s) const {
     return GP_TILE * std::min<int64_t>(GP_GROUP64, (sn_w[s] + GP_TILE - 1) / GP_TILE);
   }
@@ -392,6 +393,7 @@ struct gp_factor_s {
   int32_t* tiles_err = nullptr; // set when a bounded wait (tensor-core updates, solve tasks) ran out
   int32_t* flow_sync = nullptr; // the solve tasks' tickets and readiness flags (flow_sync_entries)
   __half* op64 = nullptr;       // GP_FP64: the digit planes of one level's large fronts, B x op64_entries
+  uint8_t* itile = nullptr;     // GP_FP64: the inverse tiles of one step as digit planes, B x max_large x 49,664 bytes
   int32_t* rho = nullptr;       // GP_FP64: the scale exponent of every row of L, B x n
   double* upd = nullptr;        // B x update_entries
   float* upd32 = nullptr;
@@ -456,6 +458,7 @@ void compute_dest_map(gp_ctx* ctx, gp_pointset* ps);
 void compute_dest_map_mixed(gp_ctx* ctx, gp_pointset* ps);
 void build_update_maps(gp_ctx* ctx, gp_factor_t* f);
 void build_digit_maps(gp_ctx* ctx, gp_factor_t* f);
+int64_t itile_bytes(const SymPlan& sp);   // of one proposal
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 int64_t bwd_part_entries(const SymPlan& sp);
 // The solve tasks' tickets (forward and backward, one each per level) and readiness flags (forward and

@@ -401,6 +401,7 @@ void build_symbolic(int64_t n, const int64_t* rowptr, const int32_t* col, const 
   sp.sn_lo_off.assign(sp.ns, 0);
   sp.sn_op64_off.assign(sp.ns, 0);
   sp.op64_entries = 64;
+  sp.max_large = 1;
   sp.lo_entries = 8;
   sp.level_large.assign(sp.nlevels, SymPlan::LevelLarge());
   sp.sn_fl.assign(sp.ns, -1);
@@ -568,6 +569,7 @@ void build_symbolic(int64_t n, const int64_t* rowptr, const int32_t* col, const 
         o64 += 6 * (int64_t)(sp.sn_w[s] + sp.sn_r[s]) * sp.op64_ldk(s);
       }
       sp.op64_entries = std::max(sp.op64_entries, o64);
+      sp.max_large = std::max<int64_t>(sp.max_large, (int64_t)large.size());
     }
     // dataflow solve tasks of this level's large fronts (SB blocks of 64 columns per chain task: 2 where the
     // level's chains are long, else 1; rows below the columns in tasks of 64 SB rows): forward tasks ordered by

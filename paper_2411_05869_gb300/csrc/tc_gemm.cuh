@@ -58,6 +58,22 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, WaitLi
   }
   return false;
 }
+// The same, acquiring at cluster scope (for arrivals from another CTA of the cluster).
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, WaitLimit lim = DEFAULT_WAIT) {
+  const uint64_t t0 = global_ns();
+  for (uint32_t it = 0; it < lim.polls; it++) {
+    uint32_t ok;
+    asm volatile(
+        "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, "
+        "p;\n}\n"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if ((it & 63) == 63 && global_ns() - t0 > lim.ns) return false;
+  }
+  return false;
+}
 // Completes `bytes` of the barrier's expected transaction count without a copy (balances an expectation that no
 // copy will meet).
 __device__ __forceinline__ void mbar_complete_tx(uint64_t* bar, uint32_t bytes) {
@@ -171,6 +187,23 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const void* tmap, int 
       "[%6];\n" ::"r"(dst),
       "l"(tmap), "r"(x), "r"(y), "r"(z), "r"(w), "r"(smem_u32(bar))
       : "memory");
+}
+
+// An untiled bulk copy of `bytes` (16-byte aligned, like both addresses) into shared memory, completing on `bar`.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_t bytes, uint64_t* bar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(smem_u32(bar))
+               : "memory");
+}
+// 4-D tiled TMA store from shared memory (elements outside the tensor are not written), and the wait of the issuing
+// thread until all its stores are done.
+__device__ __forceinline__ void tma_store_4d(const void* tmap, int x, int y, int z, int w, uint32_t src) {
+  asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];\n" ::"l"(tmap),
+               "r"(x), "r"(y), "r"(z), "r"(w), "r"(src)
+               : "memory");
+}
+__device__ __forceinline__ void bulk_store_wait() {
+  asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group 0;\n" ::: "memory");
 }
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {
