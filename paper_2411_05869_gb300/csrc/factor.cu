@@ -4,10 +4,9 @@
 // Front of supernode s: order m = w + r, rows = its w columns then the r rows below it. Its first w columns
 // are the panel (stored column-major, ld m, in the factor); the trailing r x r block is the update matrix U_s
 // (column-major, ld r, in the update workspace). Per level:
-//   1. zero the update matrices of the level's supernodes;
-//   2. extend-add: every child's update matrix is added into its parent's front through the child's
-//      relative indices, one launch per child slot so that contributions arrive in a fixed order;
-//   3. partial factorization of each front: POTRF of the w x w diagonal block, TRSM of the r rows below,
+//   1. assembly: the update matrices are zeroed and every child's update matrix is added into its parent's front
+//      through the child's relative indices, in child order (extend_add.cuh);
+//   2. partial factorization of each front: POTRF of the w x w diagonal block, TRSM of the r rows below,
 //      SYRK of U_s -= L21 L21^T. Fronts of order <= 96 are factored by one CTA in shared memory; the larger ones
 //      advance together 64 columns (a block) at a time, in groups of 4 blocks: the block's columns receive the
 //      updates of the group's earlier blocks, POTRF of the 64 x 64 diagonal tile with its inverse, the rows below
@@ -23,6 +22,7 @@
 #include <climits>
 #include <cstring>
 
+#include "extend_add.cuh"
 #include "f64_digits.cuh"
 #include "gp_internal.cuh"
 #include "potrf64.cuh"
@@ -62,36 +62,6 @@ __device__ __forceinline__ double checked_sqrt(double d, int32_t* notpd, int32_t
     return 1.0;
   }
   return sqrt(d);
-}
-
-__global__ void k_zero_updates(const int32_t* __restrict__ list, DevPlan dp, double* __restrict__ upd, int64_t UE) {
-  int32_t s = list[blockIdx.x];
-  double* U = upd + (int64_t)blockIdx.y * UE + dp.uoff[s];
-  int64_t cnt = (int64_t)dp.r[s] * dp.r[s];
-  for (int64_t t = threadIdx.x; t < cnt; t += blockDim.x) U[t] = 0.0;
-}
-
-// One CTA per (child, 8 update columns); adds U_child into the parent's front.
-__global__ void k_extend_add(const int2* __restrict__ tab, DevPlan dp, const int32_t* __restrict__ sn_parent,
-                             double* __restrict__ panels, double* __restrict__ upd, int64_t PE, int64_t UE) {
-  int2 task = tab[blockIdx.x];
-  int32_t c = task.x, c0 = task.y;
-  int b = blockIdx.y;
-  double* pan = panels + (int64_t)b * PE;
-  double* up = upd + (int64_t)b * UE;
-  int32_t p = sn_parent[c];
-  int32_t rc = dp.r[c];
-  const double* Uc = up + dp.uoff[c];
-  const int32_t* rel = dp.relidx + dp.relidx_off[c];
-  FrontRef fp = front_of(dp, p, pan, up);
-  int32_t c1 = min(c0 + 8, rc);
-  for (int32_t bc = c0; bc < c1; bc++) {
-    int32_t tc = rel[bc];
-    for (int32_t a = bc + threadIdx.x; a < rc; a += blockDim.x) {
-      int32_t tr = rel[a];
-      *front_at(fp, tr, tc) += Uc[(int64_t)bc * rc + a];
-    }
-  }
 }
 
 // Whole partial factorization of a front of order <= GP_SMALL_M in shared memory.
@@ -673,18 +643,14 @@ static void factor_body(gp_ctx* ctx, gp_factor_t* f) {
   GP_CUDA(cudaMemsetAsync(f->tiles_err, 0, sizeof(int32_t), st));
   k_row_scale<<<dim3(grid_for(ps->n, 256), B), 256, 0, st>>>(dp, ps->n, f->panels, PE, f->rho);
   GP_CHECK_LAUNCH(ctx);
-  const int32_t* d_sn_parent = dp.sn_parent;
   ProfLevelScope pls_(ctx);
   for (int32_t L = 0; L < sp.nlevels; L++) {
     const SymPlan::Level& lv = sp.levels[L];
     ctx->prof_level = L;
-    int32_t nl = sp.lev_ptr[L + 1] - sp.lev_ptr[L];
-    k_zero_updates<<<dim3(nl, B), 256, 0, st>>>(dp.lev_sn + sp.lev_ptr[L], dp, f->upd, UE);
-    GP_CHECK_LAUNCH(ctx);
-    for (const auto& ea : lv.ea) {
+    if (lv.asm_n > 0) {
       ProfScope ps_(ctx, KC_EXTEND_ADD);
-      k_extend_add<<<dim3((unsigned)ea.ncta, B), 128, 0, st>>>(dp.ea_tab + ea.tab_off, dp, d_sn_parent, f->panels,
-                                                               f->upd, PE, UE);
+      ea::k_assemble64<<<dim3((unsigned)lv.asm_n, B), ea::THREADS, 0, st>>>(dp.asm_tab + lv.asm_off, dp, f->panels,
+                                                                           f->upd, PE, UE);
       GP_CHECK_LAUNCH(ctx);
     }
     if (lv.nsmall > 0) {

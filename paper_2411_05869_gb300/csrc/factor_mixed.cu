@@ -7,8 +7,8 @@
 // contiguous, as the tensor-core operands want), FP64 diagonal tiles (tile t of s at doff + t * 4096, row-major
 // 64 x 64), FP32 update matrices (row-major r x r). Entries (i, j) of a front with i, j < w in the same 64-block
 // live in the FP64 tile, every other panel entry in FP32.
-// Per level: zero the update matrices, extend-add the children (FP32 sums into the parent's FP32 entries and
-// FP64 tiles), factor fronts of order <= 96 wholly in FP64 shared memory, and step the large fronts 64 columns
+// Per level: assembly (the update matrices zeroed, the children added in FP32 into the parent's FP32 entries and
+// FP64 tiles: extend_add.cuh), factor fronts of order <= 96 wholly in FP64 shared memory, and step the large fronts 64 columns
 // at a time: POTRF of the diagonal tile (FP64, with the FP32 inverse of its factor), TRSM of the
 // rows below in FP32, then the updates F[i, j] -= sum_l L[i, l] L[j, l] on the tensor cores (left-looking
 // 128 x 64 strips per block, 256 x 256 CTA-pair tiles at a group's end), each FP32 operand split into two FP16
@@ -23,6 +23,7 @@
 #include <cstring>
 #include <mutex>
 
+#include "extend_add.cuh"
 #include "gp_internal.cuh"
 #include "tc_gemm.cuh"
 
@@ -70,112 +71,12 @@ __device__ __forceinline__ void mix_set(const MixFront& fr, int64_t i, int64_t j
     fr.Uu[(i - fr.w) * fr.r + (j - fr.w)] = (float)v;
   }
 }
-__device__ __forceinline__ void mix_add(const MixFront& fr, int64_t i, int64_t j, float v) {
-  if (j < fr.w) {
-    if (in_diag(fr, i, j)) *diag_at(fr, i, j) += (double)v;
-    else fr.P[i * fr.ldw + j] += v;
-  } else {
-    fr.Uu[(i - fr.w) * fr.r + (j - fr.w)] += v;
-  }
-}
-
 __device__ __forceinline__ double checked_sqrt(double d, int32_t* notpd, int32_t col) {
   if (!(d > 0.0)) {
     atomicMin(notpd, col);
     return 1.0;
   }
   return sqrt(d);
-}
-
-// Row a and column b of entry e of a lower triangle stored by rows (e = a (a + 1) / 2 + b, b <= a).
-__device__ __forceinline__ void tri_decode(int64_t e, int64_t& a, int64_t& b) {
-  int64_t r = (int64_t)((sqrtf(8.f * (float)e + 1.f) - 1.f) * 0.5f);
-  while ((r + 1) * (r + 2) / 2 <= e) r++;
-  while (r * (r + 1) / 2 > e) r--;
-  a = r;
-  b = e - r * (r + 1) / 2;
-}
-
-// The update matrices' lower triangles (row a, columns b <= a; nothing reads or writes the upper ones) are zeroed
-// and extend-added in chunks of GP_EA_CHUNK entries in row order, one CTA per (supernode, chunk): every thread
-// has work however short the rows are (the small fronts' update matrices are thousands of short rows). Thread t
-// takes the chunk's entries t, t + 256, ..., EA_G of them at a time with all their loads in flight, stepping
-// (row, column) along instead of decoding every entry.
-constexpr int EA_THREADS = 256, EA_PER = GP_EA_CHUNK / EA_THREADS, EA_G = 4;
-__device__ __forceinline__ void tri_step(int64_t e, int64_t& a, int64_t& b) {   // entry e = the previous + 256
-  b += EA_THREADS;
-  if (b > a) tri_decode(e, a, b);
-}
-
-__global__ void __launch_bounds__(EA_THREADS) k_zero_updates32(const int2* __restrict__ tab, DevPlan dp,
-                                                               float* __restrict__ upd, int64_t UE) {
-  const int2 task = tab[blockIdx.x];
-  const int32_t s = task.x;
-  float* U = upd + (int64_t)blockIdx.y * UE + dp.uoff[s];
-  const int64_t r = dp.r[s], E = r * (r + 1) / 2;
-  int64_t e = (int64_t)task.y * GP_EA_CHUNK + threadIdx.x, a, b;
-  if (e >= E) return;
-  tri_decode(e, a, b);
-  for (int k = 0; k < EA_PER && e < E; k++) {
-    U[a * r + b] = 0.f;
-    e += EA_THREADS;
-    if (e < E) tri_step(e, a, b);
-  }
-}
-
-// Entries a, b <= a of the child's update matrix into the parent front (row rel[a], column rel[b]). The targets of
-// distinct entries are distinct (rel is increasing) and a launch takes one child of each parent, so no two
-// threads of a launch touch one target.
-__global__ void __launch_bounds__(EA_THREADS) k_extend_add32(const int2* __restrict__ tab, DevPlan dp,
-                                                             float* __restrict__ p32, double* __restrict__ dg,
-                                                             float* __restrict__ u32, int64_t P32E, int64_t DE,
-                                                             int64_t UE) {
-  const int2 task = tab[blockIdx.x];
-  const int32_t c = task.x;
-  const int bp = blockIdx.y;
-  float* pp = p32 + (int64_t)bp * P32E;
-  double* pd = dg + (int64_t)bp * DE;
-  float* pu = u32 + (int64_t)bp * UE;
-  const int32_t p = dp.sn_parent[c];
-  const int64_t rc = dp.r[c], E = rc * (rc + 1) / 2;
-  const float* Uc = pu + dp.uoff[c];
-  const int32_t* rel = dp.relidx + dp.relidx_off[c];
-  const MixFront fp = mix_front(dp, p, pp, pd, pu);
-  int64_t e = (int64_t)task.y * GP_EA_CHUNK + threadIdx.x, a = 0, b = 0;
-  if (e >= E) return;
-  tri_decode(e, a, b);
-  for (int k0 = 0; k0 < EA_PER && e < E; k0 += EA_G) {
-    int32_t tr[EA_G], cc[EA_G];
-    float vv[EA_G];
-#pragma unroll
-    for (int k = 0; k < EA_G; k++) {
-      tr[k] = -1;
-      if (e < E) {
-        tr[k] = rel[a];
-        cc[k] = rel[b];
-        vv[k] = Uc[a * rc + b];
-        e += EA_THREADS;
-        if (e < E) tri_step(e, a, b);
-      }
-    }
-    float old[EA_G];
-#pragma unroll
-    for (int k = 0; k < EA_G; k++)   // a row below the parent's columns: its update-matrix row or FP32 panel row
-      if (tr[k] >= fp.w)
-        old[k] = cc[k] >= fp.w ? fp.Uu[(int64_t)(tr[k] - fp.w) * fp.r + (cc[k] - fp.w)]
-                               : fp.P[(int64_t)tr[k] * fp.ldw + cc[k]];
-#pragma unroll
-    for (int k = 0; k < EA_G; k++) {
-      if (tr[k] < 0) continue;
-      if (tr[k] >= fp.w) {
-        float* t = cc[k] >= fp.w ? fp.Uu + (int64_t)(tr[k] - fp.w) * fp.r + (cc[k] - fp.w)
-                                 : fp.P + (int64_t)tr[k] * fp.ldw + cc[k];
-        *t = old[k] + vv[k];
-      } else {   // a row of the parent's columns: panel or FP64 diagonal tile
-        mix_add(fp, tr[k], cc[k], vv[k]);
-      }
-    }
-  }
 }
 
 // Fronts of order <= GP_SMALL_M: the whole partial factorization in FP64 shared memory.
@@ -1494,27 +1395,14 @@ void factor_run_mixed(gp_ctx* ctx, gp_factor_t* f) {
   GP_CUDA(cudaMemsetAsync(f->tiles_err, 0, sizeof(int32_t), st));
   ProfLevelScope pls_(ctx);
   // Work off the level chain goes to the context's side stream (not while profiling, which times every launch on
-  // the main stream): zeroing level L + 1's update matrices once level L's extend-add has read the matrices they
-  // may reuse, and the FP64 L_11 of level L's diagonal tiles once its block steps are done (nothing later touches
-  // them). The main stream waits for a level's zeroing before its extend-add, and for everything at the end.
+  // the main stream): the FP64 L_11 of level L's diagonal tiles once its block steps are done (nothing later touches
+  // them). The main stream waits for it at the end.
   const bool overlap = ctx->side != nullptr && !ctx->prof;
   const bool tiles64 = !f->diag_fp32 && !sp.large_fronts.empty();
-  auto zero_level = [&](int32_t L, cudaStream_t s) {
-    const SymPlan::Level& lz = sp.levels[L];
-    if (lz.zero_n == 0) return;
-    ProfScope ps_(ctx, KC_EXTEND_ADD);   // the update matrices this level's fronts will fill
-    k_zero_updates32<<<dim3((unsigned)lz.zero_n, B), EA_THREADS, 0, s>>>(dp.zero_tab + lz.zero_off, dp, f->upd32, UE);
-    GP_CHECK_LAUNCH(ctx);
-  };
   auto fork = [&]() {
     GP_CUDA(cudaEventRecord(ctx->ev_fork, st));
     GP_CUDA(cudaStreamWaitEvent(ctx->side, ctx->ev_fork, 0));
   };
-  if (overlap && sp.nlevels > 0) {
-    fork();
-    zero_level(0, ctx->side);
-    GP_CUDA(cudaEventRecord(ctx->ev_join, ctx->side));
-  }
   // The left-looking update of a step (mode 3, or 4 for a pair of block columns). With a third stream (explicit
   // streams, not while profiling) and at most half the SMs taken by the step's fronts, the strip's first 128-row
   // tile of each front -- the rows of the step's diagonal tiles, which the POTRF factors -- runs on the main
@@ -1540,18 +1428,11 @@ void factor_run_mixed(gp_ctx* ctx, gp_factor_t* f) {
   for (int32_t L = 0; L < sp.nlevels; L++) {
     const SymPlan::Level& lv = sp.levels[L];
     ctx->prof_level = L;
-    if (overlap) GP_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));   // this level's zeroing
-    else zero_level(L, st);
-    for (const auto& ea : lv.ea32) {
+    if (lv.asm_n > 0) {
       ProfScope ps_(ctx, KC_EXTEND_ADD);
-      k_extend_add32<<<dim3((unsigned)ea.ncta, B), EA_THREADS, 0, st>>>(dp.ea32_tab + ea.tab_off, dp, f->panels32,
-                                                                        f->diag, f->upd32, P32E, DE, UE);
+      ea::k_assemble32<<<dim3((unsigned)lv.asm_n, B), ea::THREADS, 0, st>>>(dp.asm_tab + lv.asm_off, dp, f->panels32,
+                                                                           f->diag, f->upd32, P32E, DE, UE);
       GP_CHECK_LAUNCH(ctx);
-    }
-    if (overlap && L + 1 < sp.nlevels) {   // the next level's zeroing, beside this level's steps
-      fork();
-      zero_level(L + 1, ctx->side);
-      GP_CUDA(cudaEventRecord(ctx->ev_join, ctx->side));
     }
     if (lv.nsmall > 0) {
       int32_t mmax = 1;
@@ -1627,7 +1508,7 @@ void factor_run_mixed(gp_ctx* ctx, gp_factor_t* f) {
     }
   }
   ctx->prof_level = -1;   // one launch over all levels
-  if (overlap) {
+  if (overlap && tiles64) {
     GP_CUDA(cudaEventRecord(ctx->ev_join, ctx->side));
     GP_CUDA(cudaStreamWaitEvent(st, ctx->ev_join, 0));
   } else if (tiles64) {   // L_11 of every diagonal tile in FP64

@@ -412,41 +412,30 @@ void build_symbolic(int64_t n, const int64_t* rowptr, const int32_t* col, const 
   sp.flow_bwd_ptr.assign(1, 0);
   for (int32_t L = 0; L < sp.nlevels; L++) {
     SymPlan::Level& lv = sp.levels[L];
-    // extend-add: k-th child of every supernode of this level, 8 update columns per CTA
-    int32_t maxch = 0;
-    for (int32_t q = sp.lev_ptr[L]; q < sp.lev_ptr[L + 1]; q++) {
-      int32_t s = sp.lev_sn[q];
-      maxch = std::max(maxch, sp.ch_ptr[s + 1] - sp.ch_ptr[s]);
-    }
-    for (int32_t k = 0; k < maxch; k++) {
-      SymPlan::EaLaunch ea{(int64_t)sp.ea_tab.size(), 0};
-      for (int32_t q = sp.lev_ptr[L]; q < sp.lev_ptr[L + 1]; q++) {
-        int32_t s = sp.lev_sn[q];
-        if (sp.ch_ptr[s] + k >= sp.ch_ptr[s + 1]) continue;
-        int32_t c = sp.ch_idx[sp.ch_ptr[s] + k];
-        for (int32_t c0 = 0; c0 < sp.sn_r[c]; c0 += 8) sp.ea_tab.push_back(make_int2(c, c0));
-      }
-      ea.ncta = (int64_t)sp.ea_tab.size() - ea.tab_off;
-      if (ea.ncta > 0) lv.ea.push_back(ea);
-      SymPlan::EaLaunch e32{(int64_t)sp.ea32_tab.size(), 0};
-      for (int32_t q = sp.lev_ptr[L]; q < sp.lev_ptr[L + 1]; q++) {
-        int32_t s = sp.lev_sn[q];
-        if (sp.ch_ptr[s] + k >= sp.ch_ptr[s + 1]) continue;
-        int32_t c = sp.ch_idx[sp.ch_ptr[s] + k];
-        const int64_t rc = sp.sn_r[c], nch = (rc * (rc + 1) / 2 + GP_EA_CHUNK - 1) / GP_EA_CHUNK;
-        GP_REQUIRE(nch < INT32_MAX, "update matrix too large");
-        for (int64_t h = 0; h < nch; h++) sp.ea32_tab.push_back(make_int2(c, (int)h));
-      }
-      e32.ncta = (int64_t)sp.ea32_tab.size() - e32.tab_off;
-      if (e32.ncta > 0) lv.ea32.push_back(e32);
-    }
-    lv.zero_off = (int64_t)sp.zero_tab.size();
+    // assembly: the fronts' lower triangles in runs of whole rows of about equal size, of the fronts that have children
+    // or an update matrix. About 8192 entries per run, fewer on a level with little to assemble (so that it spreads over
+    // the GPU), and at least eight rows where that leaves the level some 600 runs (the kernel takes four rows at a time;
+    // with a run of 8192 entries a front of order 25,000 has one row in each: 34.6 ms of assembly at n = 600k)
+    double level_entries = 0.0;
     for (int32_t q = sp.lev_ptr[L]; q < sp.lev_ptr[L + 1]; q++) {
       const int32_t s = sp.lev_sn[q];
-      const int64_t r = sp.sn_r[s], nch = (r * (r + 1) / 2 + GP_EA_CHUNK - 1) / GP_EA_CHUNK;
-      for (int64_t h = 0; h < nch; h++) sp.zero_tab.push_back(make_int2(s, (int)h));
+      level_entries += 0.5 * ((double)sp.sn_w[s] + sp.sn_r[s]) * ((double)sp.sn_w[s] + sp.sn_r[s]);
     }
-    lv.zero_n = (int64_t)sp.zero_tab.size() - lv.zero_off;
+    const int64_t run = std::min<int64_t>(GP_EA_CHUNK, std::max<int64_t>(GP_EA_CHUNK / 8, (int64_t)(level_entries / 1024)));
+    lv.asm_off = (int64_t)sp.asm_tab.size();
+    for (int32_t q = sp.lev_ptr[L]; q < sp.lev_ptr[L + 1]; q++) {
+      const int32_t s = sp.lev_sn[q];
+      const int32_t m = sp.sn_w[s] + sp.sn_r[s];
+      if (sp.ch_ptr[s] == sp.ch_ptr[s + 1] && sp.sn_r[s] == 0) continue;
+      for (int32_t i0 = 0; i0 < m;) {
+        int32_t i1 = i0;
+        const int32_t rows = 8.0 * 600.0 * m <= level_entries ? 8 : 1;
+        for (int64_t e = 0; i1 < m && (i1 - i0 < rows || e + i1 + 1 <= run); i1++) e += i1 + 1;
+        sp.asm_tab.push_back(make_int4(s, i0, i1, 0));
+        i0 = i1;
+      }
+    }
+    lv.asm_n = (int64_t)sp.asm_tab.size() - lv.asm_off;
     // fronts
     lv.small_off = (int64_t)sp.small_list.size();
     std::vector<int32_t> large;
