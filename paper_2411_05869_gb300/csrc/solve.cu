@@ -4,8 +4,8 @@
 // with log det C_z = 2 sum_j log L_jj.
 //
 // Forward (levels ascending): the front vector of supernode s (m entries, own columns then the rows below)
-// starts as the permuted right-hand side on its columns, receives every child's update vector through the
-// child's relative indices (children in order), then x = L11^{-1} f_1 and f_2 -= L21 x; f_2 is the update
+// starts as the permuted right-hand side on its columns (zero below), receives every child's update vector through the
+// child's relative indices (children in order; every task its own rows), then x = L11^{-1} f_1 and f_2 -= L21 x; f_2 is the update
 // vector handed to the parent. Backward (levels descending): t = x - L21^T alpha'(rows below), then
 // L11^T z = t. Fronts of order <= 96 use one CTA; the larger fronts of a level take one launch per sweep, in
 // tasks of 64 rows (forward) or 64 columns (backward) that wait for the blocks they need (k_fwd_flow,
@@ -18,6 +18,9 @@
 // the quadratic form is alpha^T (2 r - C alpha) in FP64, exact to second order in the residual, and the
 // log-determinant is summed in FP64 from the FP64 diagonal tiles.
 // Sums use fixed-shape trees, so results are bitwise reproducible.
+// A sweep is a chain of one or two launches per level: the gather of the children's vectors and the sum of the backward
+// partial sums run inside the tasks that use them (as launches of their own, 16 and 6 us per level, they made the
+// solves of a log-likelihood 0.91 ms instead of 0.71 at n = 9000, 3.00 instead of 2.56 at 100k, mixed).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -45,121 +48,170 @@ __global__ void k_rhs(const double* __restrict__ rhs, const int32_t* __restrict_
   work[(int64_t)b * ws + dp.frow_off[s] + (j - dp.sn_first[s])] = (V)rhs[(int64_t)b * n + perm[j]];
 }
 
-// Children's update vectors into the front vector of each supernode of the list: CTA (x, y, z) takes rows
-// [GATHER_ROWS y, GATHER_ROWS (y + 1)) of front list[x] for proposal z, and adds, child by child in child order,
-// the entries whose relative index falls there (rel is increasing, so they are one range per child). Every row
-// receives its children's entries in child order whatever the row split, so the sums do not depend on it.
-constexpr int GATHER_ROWS = 1024;
-__device__ __forceinline__ int32_t lower_bound_i32(const int32_t* __restrict__ a, int32_t n, int32_t key) {
-  int32_t lo = 0, hi = n;
-  while (lo < hi) {
-    const int32_t mid = (lo + hi) >> 1;
-    if (a[mid] < key) lo = mid + 1;
-    else hi = mid;
-  }
-  return lo;
-}
+// The children's update vectors on rows [r0, r0 + nr) of front s, added child by child in child order into g[0, nr)
+// (shared memory, initialised by the caller), by the whole CTA. Per child those rows are one range of its rows (rel is
+// increasing). A warp finds both ends of a child's range by a 16-way search, a half-warp each (the eight warps take
+// eight children at a time), so that finding them costs three or four dependent reads instead of a dozen.
 template <class V>
-__global__ void k_fwd_gather(const int32_t* __restrict__ list, DevPlan dp, V* __restrict__ work, int64_t ws) {
-  const int32_t s = list[blockIdx.x];
-  const int64_t m = (int64_t)dp.w[s] + dp.r[s];
-  const int64_t lo = (int64_t)blockIdx.y * GATHER_ROWS;
-  if (lo >= m) return;
-  const int32_t rlo = (int32_t)lo, rhi = (int32_t)min(m, lo + GATHER_ROWS);
-  V* W = work + (int64_t)blockIdx.z * ws;
-  V* fv = W + dp.frow_off[s];
-  __shared__ int32_t rng[2];
-  for (int32_t q = dp.ch_ptr[s]; q < dp.ch_ptr[s + 1]; q++) {
-    const int32_t c = dp.ch_idx[q];
-    const V* uc = W + dp.frow_off[c] + dp.w[c];
-    const int32_t* rel = dp.relidx + dp.relidx_off[c];
-    if (threadIdx.x < 2) rng[threadIdx.x] = lower_bound_i32(rel, dp.r[c], threadIdx.x == 0 ? rlo : rhi);
+__device__ __forceinline__ void gather_rows(const DevPlan& dp, const V* __restrict__ W, int32_t s, int64_t r0, int nr,
+                                            V* g) {
+  __shared__ int2 crng[8];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = min((int)(blockDim.x >> 5), 8);
+  const int32_t q0 = dp.ch_ptr[s], q1 = dp.ch_ptr[s + 1];
+  for (int32_t qb = q0; qb < q1; qb += nw) {
+    if (warp < nw && qb + warp < q1) {
+      const int32_t c = dp.ch_idx[qb + warp];
+      const int32_t* rel = dp.relidx + dp.relidx_off[c];
+      const int32_t key = (int32_t)r0 + (lane < 16 ? 0 : nr);
+      int32_t lo = 0, hi = dp.r[c];   // the first entry >= key is in [lo, hi]
+      while (__any_sync(0xffffffffu, lo < hi)) {
+        const int32_t step = (hi - lo + 15) >> 4;   // 0 once found
+        const int32_t p = lo + (lane & 15) * step;
+        const bool less = p < hi && rel[p] < key;
+        const int n = __popc(__ballot_sync(0xffffffffu, less) >> (lane & 16) & 0xffffu);   // probes below key
+        if (step > 0) {
+          const int32_t nlo = n > 0 ? lo + (n - 1) * step + 1 : lo;
+          hi = n < 16 ? min(hi, lo + n * step) : hi;
+          lo = nlo;
+        }
+      }
+      const int32_t other = __shfl_xor_sync(0xffffffffu, lo, 16);
+      if (lane == 0) crng[warp] = make_int2(lo, other);
+    }
     __syncthreads();
-    const int32_t a0 = rng[0], a1 = rng[1];
-    for (int32_t a = a0 + threadIdx.x; a < a1; a += blockDim.x) fv[rel[a]] += uc[a];
-    __syncthreads();   // this child's entries land before the next child's, and rng is free again
+    for (int k = 0; k < nw && qb + k < q1; k++) {
+      const int32_t c = dp.ch_idx[qb + k];
+      const V* uc = W + dp.frow_off[c] + dp.w[c];
+      const int32_t* rel = dp.relidx + dp.relidx_off[c];
+      const int2 rg = crng[k];
+      for (int32_t i = rg.x + (int32_t)threadIdx.x; i < rg.y; i += blockDim.x) g[rel[i] - r0] += uc[i];
+      __syncthreads();   // this child's entries land before the next child's, and crng is free again
+    }
   }
 }
 
-// Forward elimination of a whole (small) front by one CTA.
+// Forward elimination of a whole (small) front by one CTA of 128 threads, a row each: the children's update vectors, then
+// x_j = f_j / L_jj and f_i -= L_ij x_j, with the next columns' entries read ahead.
+constexpr int SMALL_THREADS = 128;
+static_assert(GP_SMALL_M <= SMALL_THREADS, "a thread per row of a small front");
 template <class St>
-__global__ void k_fwd_small(const int32_t* __restrict__ list, DevPlan dp, St store, typename St::V* __restrict__ work,
-                            int64_t ws, int64_t xv_off) {
+__global__ void __launch_bounds__(SMALL_THREADS) k_fwd_small(const int32_t* __restrict__ list, DevPlan dp, St store,
+                                                             typename St::V* __restrict__ work, int64_t ws,
+                                                             int64_t xv_off) {
   using V = typename St::V;
-  __shared__ V xs;
-  __shared__ V rdg[GP_SMALL_M];   // 1 / L_jj, formed in parallel ahead of the substitution
-  int32_t s = list[blockIdx.x];
-  int b = blockIdx.y;
+  constexpr int G = 8;
+  __shared__ V xs[2], g[SMALL_THREADS];
+  const int32_t s = list[blockIdx.x];
+  const int b = blockIdx.y;
   auto A = store.acc(dp, s, b);
-  V* fv = work + (int64_t)b * ws + dp.frow_off[s];
-  V* xv = work + (int64_t)b * ws + xv_off + dp.sn_first[s];
-  const int w = dp.w[s];
-  const int64_t m = (int64_t)w + dp.r[s];
-  for (int j = threadIdx.x; j < w; j += blockDim.x) rdg[j] = V(1) / A.L(j, j);
+  V* W = work + (int64_t)b * ws;
+  V* fv = W + dp.frow_off[s];
+  V* xv = W + xv_off + dp.sn_first[s];
+  const int w = dp.w[s], m = w + dp.r[s], i = threadIdx.x;
+  g[i] = i < w ? fv[i] : V(0);
   __syncthreads();
-  for (int j = 0; j < w; j++) {
-    if (threadIdx.x == 0) {
-      xs = fv[j] * rdg[j];
-      fv[j] = xs;
-      xv[j] = xs;
-    }
-    __syncthreads();
-    V x = xs;
-    for (int64_t i = j + 1 + threadIdx.x; i < m; i += blockDim.x) fv[i] -= A.L(i, j) * x;
+  for (int32_t q = dp.ch_ptr[s]; q < dp.ch_ptr[s + 1]; q++) {   // every row of a child is a row of the front
+    const int32_t c = dp.ch_idx[q];
+    const V* uc = W + dp.frow_off[c] + dp.w[c];
+    const int32_t* rel = dp.relidx + dp.relidx_off[c];
+    for (int32_t a = i; a < dp.r[c]; a += SMALL_THREADS) g[rel[a]] += uc[a];
     __syncthreads();
   }
+  V f = g[i];
+  const V rd = i < w ? V(1) / A.L(i, i) : V(0);
+  V l[G], ln[G];
+  auto load = [&](int j0, V (&v)[G]) {
+#pragma unroll
+    for (int e = 0; e < G; e++) v[e] = j0 + e < w && i > j0 + e && i < m ? (V)A.L(i, j0 + e) : V(0);
+  };
+  load(0, l);
+  for (int j0 = 0; j0 < w; j0 += G) {
+    load(j0 + G, ln);
+#pragma unroll
+    for (int e = 0; e < G; e++) {
+      const int j = j0 + e;
+      if (j < w) {
+        if (i == j) {
+          f = f * rd;
+          xs[j & 1] = f;
+          xv[j] = f;
+        }
+        __syncthreads();
+        if (i > j) f -= l[e] * xs[j & 1];
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < G; e++) l[e] = ln[e];
+  }
+  if (i < m) fv[i] = f;
 }
 
 // Backward, small fronts (one CTA each): t_j = x_j - sum_{a < r} L[w + a, j] alpha'(R_s[a]) (warp per
 // column), then L11^T z = t by substitution; z is written to alpha'.
 template <class St>
-__global__ void k_bwd_prep(const int32_t* __restrict__ list, int solve_small, DevPlan dp, St store,
-                           typename St::V* __restrict__ work, int64_t ws, int64_t apv_off, int64_t xv_off) {
+__global__ void k_bwd_prep(const int32_t* __restrict__ list, DevPlan dp, St store, typename St::V* __restrict__ work,
+                           int64_t ws, int64_t apv_off, int64_t xv_off) {
   using V = typename St::V;
-  __shared__ V zs;
-  __shared__ V rdg[GP_SMALL_M];
+  __shared__ V zs[2], t[GP_SMALL_M], av[GP_SMALL_M];
   int32_t s = list[blockIdx.x];
   int b = blockIdx.y;
   auto A = store.acc(dp, s, b);
   V* W = work + (int64_t)b * ws;
-  V* fv = W + dp.frow_off[s];
   V* apv = W + apv_off;
   const int w = dp.w[s], r = dp.r[s];
   const int32_t* R = dp.frows + dp.frow_off[s] + w;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  const int k = threadIdx.x;
+  if (k < r) av[k] = apv[R[k]];
+  const V rd = k < w ? V(1) / A.L(k, k) : V(0);
+  __syncthreads();
   for (int j = warp; j < w; j += nw) {
     V acc = 0;
-    for (int a = lane; a < r; a += 32) acc += A.L(w + a, j) * apv[R[a]];
+    for (int a = lane; a < r; a += 32) acc += A.L(w + a, j) * av[a];
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0) fv[j] = W[xv_off + dp.sn_first[s] + j] - acc;
+    if (lane == 0) t[j] = W[xv_off + dp.sn_first[s] + j] - acc;
   }
-  if (!solve_small) return;
-  for (int j = threadIdx.x; j < w; j += blockDim.x) rdg[j] = V(1) / A.L(j, j);
   __syncthreads();
   const int32_t first = dp.sn_first[s];
-  for (int j = w - 1; j >= 0; j--) {
-    if (threadIdx.x == 0) {
-      zs = fv[j] * rdg[j];
-      fv[j] = zs;
-      apv[first + j] = zs;
+  V f = k < w ? t[k] : V(0);
+  constexpr int G = 8;
+  V l[G], ln[G];
+  auto load = [&](int j0, V (&v)[G]) {   // L[j0 - e, k], the rows above the pivots j0, j0 - 1, ...
+#pragma unroll
+    for (int e = 0; e < G; e++) v[e] = j0 - e > k ? (V)A.L(j0 - e, k) : V(0);
+  };
+  load(w - 1, l);
+  for (int j0 = w - 1; j0 >= 0; j0 -= G) {
+    load(j0 - G, ln);
+#pragma unroll
+    for (int e = 0; e < G; e++) {
+      const int j = j0 - e;
+      if (j >= 0) {
+        if (k == j) {
+          f = f * rd;
+          zs[j & 1] = f;
+          apv[first + j] = f;
+        }
+        __syncthreads();
+        if (k < j) f -= l[e] * zs[j & 1];
+      }
     }
-    __syncthreads();
-    V z = zs;
-    for (int k = threadIdx.x; k < j; k += blockDim.x) fv[k] -= A.L(j, k) * z;
-    __syncthreads();
+#pragma unroll
+    for (int e = 0; e < G; e++) l[e] = ln[e];
   }
 }
 
 // Backward, large fronts: t_j = x_j - sum_a L[w + a, j] alpha'(R_s[a]) for the 64-column stripe of each task
-// (a task per (front, stripe) over all of a level's large fronts), in two launches: partial sums over chunks of
-// BP_CH rows (grid: task x chunk), then a fixed-order sum of the chunks per task.
+// (a task per (front, stripe) over all of a level's large fronts): partial sums over chunks of BP_CH rows (grid: task x
+// chunk), which the level's backward tasks add up in chunk order. A stripe's sums are at the level's number of its
+// readiness flag.
 // Row-major: 64 threads across the stripe's columns x 4 row groups, eight loads in flight per thread;
 // column-major: a warp per column.
 constexpr int BP_CH = 128;
 
 template <class St>
 __global__ void __launch_bounds__(256) k_bwd_prep_part(const int32_t* __restrict__ fronts,
-                                                       const int32_t* __restrict__ kbs, int ntask, int nch,
+                                                       const int32_t* __restrict__ kbs, int ntask, int nch, int fl0,
                                                        DevPlan dp, St store, const typename St::V* __restrict__ work,
                                                        int64_t ws, int64_t apv_off, typename St::V* __restrict__ part) {
   using V = typename St::V;
@@ -175,7 +227,7 @@ __global__ void __launch_bounds__(256) k_bwd_prep_part(const int32_t* __restrict
   const V* apv = work + (int64_t)b * ws + apv_off;
   const int nj = min(T, w - j0);
   const int32_t* R = dp.frows + dp.frow_off[s] + w;
-  V* out = part + (((int64_t)b * ntask + task) * nch + chunk) * T;
+  V* out = part + (((int64_t)b * ntask + (dp.sn_fl[s] + kbs[task] - fl0)) * nch + chunk) * T;
   if constexpr (St::kRowMajor) {
     const int c = threadIdx.x & 63, g = threadIdx.x >> 6;
     V acc = 0;
@@ -207,23 +259,6 @@ __global__ void __launch_bounds__(256) k_bwd_prep_part(const int32_t* __restrict
   }
 }
 
-template <class V>
-__global__ void k_bwd_prep_sum(const int32_t* __restrict__ fronts, const int32_t* __restrict__ kbs, int ntask,
-                               int nch, DevPlan dp, V* __restrict__ work, int64_t ws, int64_t xv_off,
-                               const V* __restrict__ part) {
-  const int task = blockIdx.x, b = blockIdx.y, c = threadIdx.x;
-  const int32_t s = fronts[task];
-  const int j0 = kbs[task] * T;
-  const int nj = min(T, dp.w[s] - j0);
-  if (c >= nj) return;
-  const int nc = (dp.r[s] + BP_CH - 1) / BP_CH;
-  const V* p = part + ((int64_t)b * ntask + task) * nch * T + c;
-  V acc = 0;
-  for (int k = 0; k < nc; k++) acc += p[(int64_t)k * T];
-  V* W = work + (int64_t)b * ws;
-  W[dp.frow_off[s] + j0 + c] = W[xv_off + dp.sn_first[s] + j0 + c] - acc;
-}
-
 // ---------------------------------------------------------------------------------------------------------
 // The large fronts of a level, one launch per sweep. Every CTA draws a ticket, the index of its task in the
 // level's task list (tasks x proposals, proposals inner), and waits (bounded) only for blocks that tasks with
@@ -232,8 +267,8 @@ __global__ void k_bwd_prep_sum(const int32_t* __restrict__ fronts, const int32_t
 //   forward task (s, i < nb): x_i = inv(L_ii) (f_i - sum_{J < i} L_iJ x_J), written to x and published (flag i);
 //   forward task (s, i >= nb): f_R -= sum_{J < nb} L_RJ x_J for the 64 rows R = w + 64 (i - nb) + [0, 64)
 //     below the front's columns (the update vector handed to the parent);
-//   backward task (s, J): z_J = inv(L_JJ)^T (t_J - sum_{I > J} L_IJ^T z_I), with t_J = x_J - L_{R,J}^T alpha'(R)
-//     as the level's partial-sum launches left it in the front vector, written to alpha' and published (flag J).
+//   backward task (s, J): z_J = inv(L_JJ)^T (t_J - sum_{I > J} L_IJ^T z_I), with t_J = x_J - L_{R,J}^T alpha'(R) from
+//     the level's partial sums, written to alpha' and published (flag J).
 // A task publishes only after it has read every block it needs, so a published flag implies all flags before it
 // (after it, backward): one acquire of the last block a task needs covers the rest once the chain has passed.
 // A task reads the L tile of its next block while it waits for the current one. Every task sums its blocks in
@@ -324,7 +359,7 @@ __global__ void __launch_bounds__(256, flow_min_blocks<typename St::V, SB>())
   const int64_t r0 = own ? (int64_t)i0 * T : (int64_t)w + (int64_t)(task.y - nbs) * (SB * T);
   const int nr = (int)imin64(SB * T, (own ? (int64_t)w : m) - r0);   // rows of the task
   const int nJ = own ? i0 : nb;
-  if (own) {   // the blocks' inverses, the tile between them and f, staged while the earlier blocks arrive
+  if (own) {   // the blocks' inverses and the tile between them, staged while the earlier blocks arrive
     for (int k = 0; k < nblk; k++) {
       const V* inv = store.inv(dp, s, b) + (int64_t)(i0 + k) * T * T;
       V* Ms = k == 0 ? Ms0 : Ms1;
@@ -342,8 +377,11 @@ __global__ void __launch_bounds__(256, flow_min_blocks<typename St::V, SB>())
         Tl[q * FS + l] = T + q < nr ? (V)A.L(r0 + T + q, (int64_t)i0 * T + l) : V(0);
       }
     }
-    if (threadIdx.x < SB * T) fsh[threadIdx.x] = threadIdx.x < nr ? fv[r0 + threadIdx.x] : V(0);
   }
+  // the rows' right-hand side and the children's update vectors on them
+  if (threadIdx.x < SB * T) fsh[threadIdx.x] = own && threadIdx.x < nr ? fv[r0 + threadIdx.x] : V(0);
+  __syncthreads();
+  gather_rows(dp, W, s, r0, nr, fsh);
   int ready = -1;   // blocks [0, ready] are known published
   auto need = [&](int J) {   // one acquire also covers the next 8 blocks when they are already out
     if (J <= ready) return;
@@ -431,7 +469,7 @@ __global__ void __launch_bounds__(256, flow_min_blocks<typename St::V, SB>())
   }
   __syncthreads();
   if (!own) {
-    if (threadIdx.x < nr) fv[r0 + threadIdx.x] -= tots[threadIdx.x];
+    if (threadIdx.x < nr) fv[r0 + threadIdx.x] = fsh[threadIdx.x] - tots[threadIdx.x];
     return;
   }
   // block i0
@@ -468,7 +506,8 @@ __global__ void __launch_bounds__(256, flow_min_blocks<typename St::V, SB>())
 template <class St, int SB>
 __global__ void __launch_bounds__(256, flow_min_blocks<typename St::V, SB>())
     k_bwd_flow(const int2* __restrict__ tasks, int B, DevPlan dp, St store, typename St::V* __restrict__ work,
-               int64_t ws, int64_t apv_off, int32_t* __restrict__ ticket, int32_t* __restrict__ flags, int64_t nfl,
+               int64_t ws, int64_t apv_off, int64_t xv_off, const typename St::V* __restrict__ part_sums, int ntask,
+               int nch, int fl0, int32_t* __restrict__ ticket, int32_t* __restrict__ flags, int64_t nfl,
                int32_t* __restrict__ err, tcg::WaitLimit lim) {
   using V = typename St::V;
   extern __shared__ __align__(16) unsigned char flow_sh[];
@@ -485,7 +524,6 @@ __global__ void __launch_bounds__(256, flow_min_blocks<typename St::V, SB>())
   const int J0 = task.y * SB;
   auto A = store.acc(dp, s, b);
   V* W = work + (int64_t)b * ws;
-  V* fv = W + dp.frow_off[s];
   V* zs = W + apv_off + dp.sn_first[s];   // alpha' on the front's columns
   const int w = dp.w[s];
   const int nb = (w + T - 1) / T;
@@ -510,7 +548,18 @@ __global__ void __launch_bounds__(256, flow_min_blocks<typename St::V, SB>())
       Tl[l * FS + q] = l < bw1 ? (V)A.L((int64_t)c0 + T + l, c0 + q) : V(0);
     }
   }
-  if (threadIdx.x < SB * T) tsh[threadIdx.x] = threadIdx.x < nc ? fv[c0 + threadIdx.x] : V(0);
+  if (threadIdx.x < SB * T) {   // t = x less the rows below the columns (their partial sums in chunk order)
+    V t = 0;
+    if (threadIdx.x < nc) {
+      const V* p = part_sums + ((int64_t)b * ntask + (dp.sn_fl[s] - fl0 + J0 + (threadIdx.x >> 6))) * nch * T + (threadIdx.x & 63);
+      const int n = (dp.r[s] + BP_CH - 1) / BP_CH;
+      V acc = 0;
+#pragma unroll 8
+      for (int k = 0; k < n; k++) acc += p[(int64_t)k * T];
+      t = W[xv_off + dp.sn_first[s] + c0 + threadIdx.x] - acc;
+    }
+    tsh[threadIdx.x] = t;
+  }
   const int Itop = J0 + nblk;   // the blocks above the task: I = nb - 1 down to Itop
   int ready = nb;               // blocks [ready, nb) are known published
   auto need = [&](int I) {      // one acquire also covers the next 8 blocks when they are already out
@@ -842,7 +891,6 @@ void solve_impl(gp_ctx* ctx, gp_factor_t* f, const St& store, const double* rhs,
   const int64_t xv_off = apv_off + n;
   using V = typename St::V;
   V* work = reinterpret_cast<V*>(f->work);   // ws entries of V per proposal
-  GP_CUDA(cudaMemsetAsync(f->work, 0, sizeof(V) * (size_t)B * ws, st));
   // tickets and readiness flags of the large fronts' tasks
   GP_CUDA(cudaMemsetAsync(f->flow_sync, 0, sizeof(int32_t) * (size_t)flow_sync_entries(sp, B), st));
   int32_t* fwd_flags = f->flow_sync + 2 * sp.nlevels;
@@ -853,20 +901,9 @@ void solve_impl(gp_ctx* ctx, gp_factor_t* f, const St& store, const double* rhs,
   GP_CHECK_LAUNCH(ctx);
   for (int32_t L = 0; L < sp.nlevels; L++) {
     const SymPlan::Level& lv = sp.levels[L];
-    int32_t nl = sp.lev_ptr[L + 1] - sp.lev_ptr[L];
-    if (L > 0) {
-      int64_t mmax = 1;   // row chunks of the level's largest front
-      for (int32_t q = sp.lev_ptr[L]; q < sp.lev_ptr[L + 1]; q++) {
-        const int32_t s = sp.lev_sn[q];
-        mmax = std::max<int64_t>(mmax, (int64_t)sp.sn_w[s] + sp.sn_r[s]);
-      }
-      const unsigned nch = (unsigned)((mmax + GATHER_ROWS - 1) / GATHER_ROWS);
-      k_fwd_gather<<<dim3(nl, nch, B), 256, 0, st>>>(dp.lev_sn + sp.lev_ptr[L], dp, work, ws);
-      GP_CHECK_LAUNCH(ctx);
-    }
     if (lv.nsmall > 0) {
-      k_fwd_small<St><<<dim3(lv.nsmall, B), 128, 0, st>>>(dp.small_list + lv.small_off, dp, store, work, ws,
-                                                          xv_off);
+      k_fwd_small<St><<<dim3(lv.nsmall, B), SMALL_THREADS, 0, st>>>(dp.small_list + lv.small_off, dp, store, work, ws,
+                                                                    xv_off);
       GP_CHECK_LAUNCH(ctx);
     }
     const int64_t nt = sp.flow_fwd_ptr[L + 1] - sp.flow_fwd_ptr[L];
@@ -886,26 +923,24 @@ void solve_impl(gp_ctx* ctx, gp_factor_t* f, const St& store, const double* rhs,
   for (int32_t L = sp.nlevels - 1; L >= 0; L--) {
     const SymPlan::Level& lv = sp.levels[L];
     if (lv.nsmall > 0) {
-      k_bwd_prep<St><<<dim3(lv.nsmall, B), 256, 0, st>>>(dp.small_list + lv.small_off, 1, dp, store, work, ws,
-                                                         apv_off, xv_off);
+      k_bwd_prep<St><<<dim3(lv.nsmall, B), 256, 0, st>>>(dp.small_list + lv.small_off, dp, store, work, ws, apv_off,
+                                                         xv_off);
       GP_CHECK_LAUNCH(ctx);
     }
     if (!lv.steps.empty()) {
       const auto& ll = sp.level_large[L];   // one task per (large front, 64-column stripe)
       const int nch = bwd_chunks(sp, L);
       V* part = reinterpret_cast<V*>(f->bwd_part);
+      const int fl0 = sp.sn_fl[sp.large_fronts[ll.off]];   // the level's first flag (its widest front's)
       k_bwd_prep_part<St><<<dim3((unsigned)ll.count, nch, B), 256, 0, st>>>(
-          dp.large_fronts + ll.off, dp.large_kb + ll.off, (int)ll.count, nch, dp, store, work, ws, apv_off, part);
-      GP_CHECK_LAUNCH(ctx);
-      k_bwd_prep_sum<V><<<dim3((unsigned)ll.count, B), T, 0, st>>>(dp.large_fronts + ll.off, dp.large_kb + ll.off,
-                                                                   (int)ll.count, nch, dp, work, ws, xv_off, part);
+          dp.large_fronts + ll.off, dp.large_kb + ll.off, (int)ll.count, nch, fl0, dp, store, work, ws, apv_off, part);
       GP_CHECK_LAUNCH(ctx);
       const int64_t nt = sp.flow_bwd_ptr[L + 1] - sp.flow_bwd_ptr[L];
       const auto kb = lv.flow_sb == 2 ? k_bwd_flow<St, 2> : k_bwd_flow<St, 1>;
       const size_t sm = lv.flow_sb == 2 ? flow_smem_bytes<V, 2>() : flow_smem_bytes<V, 1>();
       kb<<<(unsigned)(nt * B), 256, sm, st>>>(dp.flow_bwd + sp.flow_bwd_ptr[L], B, dp, store, work, ws, apv_off,
-                                              f->flow_sync + 2 * L + 1, bwd_flags, sp.n_fl, f->tiles_err,
-                                              f->wait_lim);
+                                              xv_off, part, (int)ll.count, nch, fl0, f->flow_sync + 2 * L + 1,
+                                              bwd_flags, sp.n_fl, f->tiles_err, f->wait_lim);
       GP_CHECK_LAUNCH(ctx);
     }
   }
