@@ -11,9 +11,9 @@
 //   zero / scatter: the active supernodes' front vectors (m_s x R) cleared, then c_k written at its neighbours'
 //         rows;
 //   levels ascending: children's update vectors added into the parents (in child order), fronts of order <= 96
-//         eliminated by one CTA, larger fronts 64 columns per launch: every CTA forms X_J = inv(L_JJ) F_J for
-//         its front (a 64 x 64 by 64 x R product) and either stores X_J (the entries of w) or applies
-//         F_I -= L_IJ X_J to one 64-row tile below; inactive (front, chunk) pairs return at once;
+//         eliminated by one CTA, larger fronts 64 columns per launch: X_0 = inv(L_00) F_0 for every front, then per
+//         block column J a CTA per 64-row tile below applies F_I -= L_IJ X_J for two chunks side by side, and the one
+//         whose rows are the next block forms X_{J+1} from them; inactive (front, chunk) pairs are left out;
 //   sum: |w_k|^2 over all entries in a fixed order, var_k = prior_k - |w_k|^2.
 // The arithmetic is the factor's working precision: FP64 with the FP64 factor; FP32 vectors with the mixed
 // factor's FP32 panels and inverses (the variance then carries the mixed factor's ~1e-6 relative accuracy).
@@ -104,13 +104,17 @@ __global__ void k_var_scatter(const double* __restrict__ Xt, int64_t m, int64_t 
   });
 }
 
-// Children's update vectors into the front vectors of the level's supernodes (children in order).
+// Children's update vectors into the front vectors of the level's supernodes (children in order): CTA (x, y, z) takes
+// rows [GROWS z, GROWS (z + 1)) of front list[x] for chunk y.
+constexpr int GROWS = 256;
 template <class V>
 __global__ void k_var_gather(const int32_t* __restrict__ list, DevPlan dp, VarWork<V> vw) {
   const int32_t s = list[blockIdx.x];
   const int c = blockIdx.y;
   const uint8_t* act = vw.active + c * vw.ns;
-  if (!act[s]) return;
+  const int32_t lo = (int32_t)blockIdx.z * GROWS;
+  if (lo >= dp.w[s] + dp.r[s] || !act[s]) return;
+  __shared__ int32_t rng[2];
   V* W = vw.F + c * vw.cs;
   V* fv = W + dp.frow_off[s] * R;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -119,8 +123,19 @@ __global__ void k_var_gather(const int32_t* __restrict__ list, DevPlan dp, VarWo
     if (!act[ch]) continue;
     const V* uc = W + ((int64_t)dp.frow_off[ch] + dp.w[ch]) * R;
     const int32_t* rel = dp.relidx + dp.relidx_off[ch];
-    for (int32_t a = warp; a < dp.r[ch]; a += nw) fv[(int64_t)rel[a] * R + lane] += uc[(int64_t)a * R + lane];
+    if (threadIdx.x < 2) {   // the child's rows that fall into this CTA's: rel is increasing
+      const int32_t key = lo + (threadIdx.x == 0 ? 0 : GROWS);
+      int32_t x = 0, y = dp.r[ch];
+      while (x < y) {
+        const int32_t mid = (x + y) >> 1;
+        if (rel[mid] < key) x = mid + 1;
+        else y = mid;
+      }
+      rng[threadIdx.x] = x;
+    }
     __syncthreads();
+    for (int32_t a = rng[0] + warp; a < rng[1]; a += nw) fv[(int64_t)rel[a] * R + lane] += uc[(int64_t)a * R + lane];
+    __syncthreads();   // this child's rows land before the next child's, and rng is free again
   }
 }
 
@@ -154,74 +169,140 @@ __global__ void k_var_small(const int32_t* __restrict__ list, DevPlan dp, St sto
   for (int e = threadIdx.x; e < (m - w) * R; e += blockDim.x) fv[(int64_t)w * R + e] = Fs[w + e / R][e % R];
 }
 
-// Block column kb of the large fronts of a step: tasks [0, nfront) store X_J = inv(L_JJ) F_J (the w entries of
-// the block's columns), the rest (the tile prefix of the rows below) apply F_I -= L_IJ X_J to one 64-row tile.
-// 256 threads; thread t forms 8 entries of its row (t >> 2) and right-hand sides 8 (t & 3) .. + 7.
+// The large fronts of a level, two chunks (CR = 64 right-hand sides) per CTA of 256 threads, a thread four rows by four
+// right-hand sides: per step of the products it reads two 16-byte vectors from shared memory for 16 multiply-adds, so
+// the products run at the FP32 (FP64) rate. (One chunk per CTA, eight entries of one row per thread, and X_J formed anew
+// by every CTA of the step: 48 ms for 2048 test points of the 100k workload's mixed factor.) Every entry's sum runs over
+// the block's columns in order.
+constexpr int CR = 2 * R;
+constexpr int MS = T + 4;   // row stride of the matrix tile in shared memory (16-byte vectors)
+template <class V>
+constexpr size_t var_step_smem() { return (size_t)(T * MS + T * CR) * sizeof(V); }
+
+// acc[e][f] = sum_{l < kl} Mt[l][tr + e] Fb[l][tc + f].
+template <class V>
+__device__ __forceinline__ void var_product(const V* Mt, const V* Fb, int kl, int tr, int tc, V (&acc)[4][4]) {
+#pragma unroll
+  for (int e = 0; e < 4; e++)
+#pragma unroll
+    for (int f = 0; f < 4; f++) acc[e][f] = V(0);
+  for (int l = 0; l < kl; l++) {
+    V a[4], x[4];
+#pragma unroll
+    for (int e = 0; e < 4; e++) a[e] = Mt[l * MS + tr + e];
+#pragma unroll
+    for (int f = 0; f < 4; f++) x[f] = Fb[l * CR + tc + f];
+#pragma unroll
+    for (int e = 0; e < 4; e++)
+#pragma unroll
+      for (int f = 0; f < 4; f++) acc[e][f] += a[e] * x[f];
+  }
+}
+
+// X_J = inv(L_JJ) F_J of block kb from Fb (F_J, zero past bw), stored for the active chunks. Mt: scratch.
+template <class St>
+__device__ __forceinline__ void var_block_solve(const typename St::V* inv, const typename St::V* Fb, typename St::V* Mt,
+                                                typename St::V* xv, bool act, int bw, int tr, int tc) {
+  using V = typename St::V;
+  for (int e = threadIdx.x; e < T * T; e += 256) Mt[(e & 63) * MS + (e >> 6)] = inv[e];   // zero past bw
+  __syncthreads();
+  V acc[4][4];
+  var_product(Mt, Fb, T, tr, tc, acc);
+  if (act) {
+#pragma unroll
+    for (int e = 0; e < 4; e++)
+      if (tr + e < bw) {
+#pragma unroll
+        for (int f = 0; f < 4; f++) xv[(int64_t)(tr + e) * R + f] = acc[e][f];
+      }
+  }
+}
+
+// This thread's rows and right-hand sides of the CTA's two chunks, and their chunk.
+template <class V>
+struct VarLane {
+  int tr, tc, c, r;   // rows tr.. +3, columns tc.. +3 of the pair = right-hand sides r.. +3 of chunk c
+  bool act;
+  V *F, *X;           // the chunk's front vectors and w entries
+  __device__ __forceinline__ VarLane(const VarWork<V>& vw, int32_t s, int nc)
+      : tr((threadIdx.x >> 4) * 4), tc((threadIdx.x & 15) * 4), c(2 * blockIdx.y + (tc >> 5)), r(tc & 31) {
+    act = c < nc && vw.active[c * vw.ns + s];
+    F = vw.F + c * vw.cs;
+    X = vw.X + c * vw.cs;
+  }
+};
+
+// X_0 of the level's large fronts.
+template <class St>
+__global__ void __launch_bounds__(256) k_var_first(const int32_t* __restrict__ fronts, int nc, DevPlan dp, St store,
+                                                   int b, VarWork<typename St::V> vw) {
+  using V = typename St::V;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  V* Mt = reinterpret_cast<V*>(smem_raw);
+  V* Fb = Mt + T * MS;
+  const int32_t s = fronts[blockIdx.x];
+  const VarLane<V> t(vw, s, nc);
+  if (!__syncthreads_or(t.act)) return;
+  const int bw = min(T, dp.w[s]);
+  const V* fv = t.F + dp.frow_off[s] * R;
+#pragma unroll
+  for (int e = 0; e < 4; e++)
+#pragma unroll
+    for (int f = 0; f < 4; f++)
+      Fb[(t.tr + e) * CR + t.tc + f] = t.act && t.tr + e < bw ? fv[(int64_t)(t.tr + e) * R + t.r + f] : V(0);
+  var_block_solve<St>(store.inv(dp, s, b), Fb, Mt, t.X + (int64_t)dp.sn_first[s] * R + t.r, t.act, bw, t.tr, t.tc);
+}
+
+// Block column kb of the large fronts of a step: F_I -= L_IJ X_J on the 64-row tiles below (pre: their prefix), and
+// X_{J+1} by the tile of the next block's rows.
 template <class St>
 __global__ void __launch_bounds__(256) k_var_step(const int32_t* __restrict__ fronts, const int64_t* __restrict__ pre,
-                                                  int nfront, int kb, DevPlan dp, St store, int b,
+                                                  int nfront, int kb, int nc, DevPlan dp, St store, int b,
                                                   VarWork<typename St::V> vw) {
   using V = typename St::V;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* Mt = reinterpret_cast<V*>(smem_raw);   // Mt[l][i]: inv[i][l], then L[r0 + i][c0 + l]   (64 x 65)
-  V* Fb = Mt + T * (T + 1);                 // Fb[l][r]: F_J, then X_J                            (64 x R)
-  const int64_t t = blockIdx.x;
-  const bool writer = t < nfront;
-  const int fi = writer ? (int)t : find_front(pre, nfront, t - nfront);
+  V* Mt = reinterpret_cast<V*>(smem_raw);   // Mt[l][i]: L[r0 + i][c0 + l]
+  V* Fb = Mt + T * MS;                      // Fb[l][r]: X_J
+  const int fi = find_front(pre, nfront, blockIdx.x);
   const int32_t s = fronts[fi];
-  const int c = blockIdx.y;
-  if (!vw.active[c * vw.ns + s]) return;
+  const VarLane<V> t(vw, s, nc);
+  if (!__syncthreads_or(t.act)) return;
   auto A = store.acc(dp, s, b);
-  V* fv = vw.F + c * vw.cs + dp.frow_off[s] * R;
   const int w = dp.w[s];
   const int64_t m = (int64_t)w + dp.r[s];
   const int c0 = kb * T, bw = min(T, w - c0), c1 = c0 + bw;
-  const V* inv = store.inv(dp, s, b) + (int64_t)kb * T * T;
-  for (int e = threadIdx.x; e < T * T; e += 256) Mt[(e & 63) * (T + 1) + (e >> 6)] = inv[e];   // zero past bw
-  for (int e = threadIdx.x; e < T * R; e += 256) {
-    const int l = e / R;
-    Fb[e] = l < bw ? fv[(int64_t)(c0 + l) * R + (e % R)] : V(0);
-  }
-  __syncthreads();
-  const int ti = threadIdx.x >> 2, tr = (threadIdx.x & 3) * 8;
-  V acc[8];
-#pragma unroll
-  for (int e = 0; e < 8; e++) acc[e] = V(0);
-  for (int l = 0; l < T; l++) {
-    const V a = Mt[l * (T + 1) + ti];
-#pragma unroll
-    for (int e = 0; e < 8; e++) acc[e] += a * Fb[l * R + tr + e];
-  }
-  __syncthreads();   // every thread has read F_J and the inverse
-#pragma unroll
-  for (int e = 0; e < 8; e++) Fb[ti * R + tr + e] = ti < bw ? acc[e] : V(0);   // X_J
-  if (writer) {
-    if (ti < bw) {
-      V* xv = vw.X + c * vw.cs + ((int64_t)dp.sn_first[s] + c0 + ti) * R;
-#pragma unroll
-      for (int e = 0; e < 8; e++) xv[tr + e] = acc[e];
-    }
-    return;
-  }
-  const int64_t r0 = c1 + (t - nfront - pre[fi]) * T;
+  const int64_t r0 = c1 + ((int64_t)blockIdx.x - pre[fi]) * T;
   const int nr = (int)imin64(T, m - r0);
-  for (int e = threadIdx.x; e < T * T; e += 256) {   // L[r0 + i][c0 + l] -> Mt[l][i], reads along the storage
+  const V* xj = t.X + ((int64_t)dp.sn_first[s] + c0) * R + t.r;
+#pragma unroll
+  for (int e = 0; e < 4; e++)
+#pragma unroll
+    for (int f = 0; f < 4; f++)
+      Fb[(t.tr + e) * CR + t.tc + f] = t.act && t.tr + e < bw ? xj[(int64_t)(t.tr + e) * R + f] : V(0);
+  for (int e = threadIdx.x; e < T * T; e += 256) {   // reads along the storage
     const int i = St::kRowMajor ? e >> 6 : e & 63, l = St::kRowMajor ? e & 63 : e >> 6;
-    Mt[l * (T + 1) + i] = (i < nr && l < bw) ? (V)A.L(r0 + i, c0 + l) : V(0);
+    Mt[l * MS + i] = (i < nr && l < bw) ? (V)A.L(r0 + i, c0 + l) : V(0);
   }
   __syncthreads();
+  V acc[4][4];
+  var_product(Mt, Fb, bw, t.tr, t.tc, acc);
+  V* row = t.F + (dp.frow_off[s] + r0 + t.tr) * R + t.r;
 #pragma unroll
-  for (int e = 0; e < 8; e++) acc[e] = V(0);
-  for (int l = 0; l < bw; l++) {
-    const V a = Mt[l * (T + 1) + ti];
+  for (int e = 0; e < 4; e++)
 #pragma unroll
-    for (int e = 0; e < 8; e++) acc[e] += a * Fb[l * R + tr + e];
-  }
-  if (ti < nr) {
-    V* row = fv + (r0 + ti) * R + tr;
+    for (int f = 0; f < 4; f++) {
+      acc[e][f] = t.act && t.tr + e < nr ? row[(int64_t)e * R + f] - acc[e][f] : V(0);
+      if (t.act && t.tr + e < nr) row[(int64_t)e * R + f] = acc[e][f];
+    }
+  if (r0 != c1 || c1 >= w) return;   // the next block's rows: its X as well
+  const int bw2 = min(T, w - c1);
+  __syncthreads();   // every thread has read X_J and the tile
 #pragma unroll
-    for (int e = 0; e < 8; e++) row[e] -= acc[e];
-  }
+  for (int e = 0; e < 4; e++)
+#pragma unroll
+    for (int f = 0; f < 4; f++) Fb[(t.tr + e) * CR + t.tc + f] = t.tr + e < bw2 ? acc[e][f] : V(0);
+  var_block_solve<St>(store.inv(dp, s, b) + (int64_t)(kb + 1) * T * T, Fb, Mt,
+                      t.X + ((int64_t)dp.sn_first[s] + c1) * R + t.r, t.act, bw2, t.tr, t.tc);
 }
 
 // Partial sums of w^2 per (chunk, right-hand side) over column slices, in a fixed order: CTA g of chunk c sums
@@ -291,9 +372,10 @@ void variance_impl(gp_ctx* ctx, gp_factor_t* f, const St& store, int b, const do
   const double* theta = f->theta_dev + (int64_t)b * f->theta_stride;
   const double* Fb = f->F + (int64_t)b * n * h0.n1;
   const double* Cb = f->Cpt ? f->Cpt + (int64_t)b * n * 2 : nullptr;
-  const size_t step_smem = (size_t)(T * (T + 1) + T * R) * sizeof(V);
+  const size_t step_smem = var_step_smem<V>();
   static_assert(sizeof(V) == 4 || sizeof(V) == 8, "working type");
   GP_CUDA(cudaFuncSetAttribute(k_var_step<St>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step_smem));
+  GP_CUDA(cudaFuncSetAttribute(k_var_first<St>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step_smem));
   ProfScope ps_(ctx, KC_PREDICT);
   for (int64_t k0 = 0; k0 < m; k0 += (int64_t)NC * R) {
     const int64_t cnt = std::min<int64_t>(m - k0, (int64_t)NC * R);
@@ -314,16 +396,26 @@ void variance_impl(gp_ctx* ctx, gp_factor_t* f, const St& store, int b, const do
       const SymPlan::Level& lv = sp.levels[L];
       const int32_t nl = sp.lev_ptr[L + 1] - sp.lev_ptr[L];
       if (L > 0) {
-        k_var_gather<V><<<dim3(nl, nc), 256, 0, st>>>(dp.lev_sn + sp.lev_ptr[L], dp, vw);
+        int32_t mmax = 1;   // the level's largest front
+        for (int32_t q = sp.lev_ptr[L]; q < sp.lev_ptr[L + 1]; q++)
+          mmax = std::max(mmax, sp.sn_w[sp.lev_sn[q]] + sp.sn_r[sp.lev_sn[q]]);
+        k_var_gather<V><<<dim3(nl, nc, (mmax + GROWS - 1) / GROWS), 256, 0, st>>>(dp.lev_sn + sp.lev_ptr[L], dp, vw);
         GP_CHECK_LAUNCH(ctx);
       }
       if (lv.nsmall > 0) {
         k_var_small<St><<<dim3(lv.nsmall, nc), 256, 0, st>>>(dp.small_list + lv.small_off, dp, store, b, vw);
         GP_CHECK_LAUNCH(ctx);
       }
+      const unsigned ncp = (unsigned)((nc + 1) / 2);   // pairs of chunks
+      if (!lv.steps.empty()) {
+        k_var_first<St><<<dim3(lv.steps[0].nfront, ncp), 256, step_smem, st>>>(dp.large_fronts + lv.steps[0].fr_off, nc,
+                                                                              dp, store, b, vw);
+        GP_CHECK_LAUNCH(ctx);
+      }
       for (const auto& stp : lv.steps) {
-        k_var_step<St><<<dim3((unsigned)(stp.nfront + stp.trsm_total), nc), 256, step_smem, st>>>(
-            dp.large_fronts + stp.fr_off, dp.step_pre + stp.pre_off, stp.nfront, stp.kb, dp, store, b, vw);
+        if (stp.trsm_total == 0) continue;
+        k_var_step<St><<<dim3((unsigned)stp.trsm_total, ncp), 256, step_smem, st>>>(
+            dp.large_fronts + stp.fr_off, dp.step_pre + stp.pre_off, stp.nfront, stp.kb, nc, dp, store, b, vw);
         GP_CHECK_LAUNCH(ctx);
       }
     }
