@@ -15,6 +15,7 @@ struct AccF64 {
   int64_t m;
   __device__ __forceinline__ double L(int64_t i, int64_t j) const { return P[j * m + i]; }
   __device__ __forceinline__ double Ld(int64_t i, int64_t j) const { return P[j * m + i]; }
+  __device__ __forceinline__ double off(int64_t i, int64_t j) const { return P[j * m + i]; }   // off the diagonal blocks
 };
 struct AccMix {
   const float* P;
@@ -28,6 +29,7 @@ struct AccMix {
     if (i < w && (i >> 6) == (j >> 6)) return (float)D[(i >> 6) * (T * T) + (i & 63) * T + (j & 63)];
     return P[i * ldw + j];
   }
+  __device__ __forceinline__ float off(int64_t i, int64_t j) const { return P[i * ldw + j]; }   // off the diagonal blocks
 };
 // The solve's working precision V: FP64 with the FP64 factor; FP32 with the mixed factor, whose solves only
 // precondition the FP64 refinement (the FP64 residual fixes the accuracy of alpha).

@@ -11,13 +11,18 @@
 //   zero / scatter: the active supernodes' front vectors (m_s x R) cleared, then c_k written at its neighbours'
 //         rows;
 //   levels ascending: children's update vectors added into the parents (in child order), fronts of order <= 96
-//         eliminated by one CTA, larger fronts 64 columns per launch: X_0 = inv(L_00) F_0 for every front, then per
-//         block column J a CTA per 64-row tile below applies F_I -= L_IJ X_J for two chunks side by side, and the one
-//         whose rows are the next block forms X_{J+1} from them; inactive (front, chunk) pairs are left out;
+//         eliminated by one CTA, larger fronts of the mixed factor by groups of four 64-column blocks J: one CTA
+//         solves a group's X_J = inv(L_JJ) (F_J - sum of the group's L_JK X_K), then one launch applies
+//         F_I -= L_IJ X_J to the later blocks' rows; a last launch applies all J to the rows below the front's
+//         columns. A CTA takes two or four of the chunks that are active in its front. FP64: a block at a time, 16 rows
+//         of one chunk per CTA;
 //   sum: |w_k|^2 over all entries in a fixed order, var_k = prior_k - |w_k|^2.
 // The arithmetic is the factor's working precision: FP64 with the FP64 factor; FP32 vectors with the mixed
 // factor's FP32 panels and inverses (the variance then carries the mixed factor's ~1e-6 relative accuracy).
+#include <cuda_pipeline.h>
+
 #include <algorithm>
+#include <type_traits>
 
 #include "factor_access.cuh"
 #include "gp_internal.cuh"
@@ -27,7 +32,6 @@ namespace {
 
 constexpr int T = GP_TILE;
 constexpr int R = 32;   // test points per chunk
-using fa::find_front;
 
 // Per chunk c: front vectors at F + c * cs (row i of front s at (frow_off[s] + i) * R), then the w entries of the
 // n permuted columns at X + c * cs (column j at j * R).
@@ -169,140 +173,271 @@ __global__ void k_var_small(const int32_t* __restrict__ list, DevPlan dp, St sto
   for (int e = threadIdx.x; e < (m - w) * R; e += blockDim.x) fv[(int64_t)w * R + e] = Fs[w + e / R][e % R];
 }
 
-// The large fronts of a level, two chunks (CR = 64 right-hand sides) per CTA of 256 threads, a thread four rows by four
-// right-hand sides: per step of the products it reads two 16-byte vectors from shared memory for 16 multiply-adds, so
-// the products run at the FP32 (FP64) rate. (One chunk per CTA, eight entries of one row per thread, and X_J formed anew
-// by every CTA of the step: 48 ms for 2048 test points of the 100k workload's mixed factor.) Every entry's sum runs over
-// the block's columns in order.
-constexpr int CR = 2 * R;
+// The large fronts of a level with the mixed factor. A CTA of 256 threads takes CH of the chunks that are active in its
+// front (32 CH right-hand sides) and a 64-row tile, a thread four rows by 2 CH right-hand sides in groups of four: per
+// step of the products it reads 1 + CH / 2 16-byte vectors from shared memory, a step ahead, for 8 CH multiply-adds. The
+// products bound it: FP32 multiply-adds, at about 60% of their rate on the wide levels, and one CTA's latency on the
+// narrow ones. The front vectors move through memory once per group of blocks, not once per block. 2048 test points of
+// the 100k workload: 48 ms with one chunk per CTA, eight entries of one row per thread and X_J formed anew by every tile
+// of a block column; 22 ms with two chunks and X_J formed once; 16.5 ms with the rows below the columns in one launch,
+// groups of four blocks and every load on its way before the first wait; 14.1 ms with the products' reads a step ahead.
+// Every entry's sum runs over a block's columns in order, and the blocks' sums are subtracted in order.
 constexpr int MS = T + 4;   // row stride of the matrix tile in shared memory (16-byte vectors)
-template <class V>
-constexpr size_t var_step_smem() { return (size_t)(T * MS + T * CR) * sizeof(V); }
+constexpr size_t var_smem(int bufs, int ch) { return (size_t)(T * MS + bufs * T * ch * R) * sizeof(float); }
 
-// acc[e][f] = sum_{l < kl} Mt[l][tr + e] Fb[l][tc + f].
-template <class V>
-__device__ __forceinline__ void var_product(const V* Mt, const V* Fb, int kl, int tr, int tc, V (&acc)[4][4]) {
+__device__ __forceinline__ void ld4(const float* p, float* d) {
+  const float4 u = *reinterpret_cast<const float4*>(p);
+  d[0] = u.x, d[1] = u.y, d[2] = u.z, d[3] = u.w;
+}
+__device__ __forceinline__ void st4(float* p, const float* d) {
+  *reinterpret_cast<float4*>(p) = make_float4(d[0], d[1], d[2], d[3]);
+}
+__device__ __forceinline__ void ld4_or_zero(bool on, const float* p, float* d) {
+  if (on) ld4(p, d);
+  else d[0] = d[1] = d[2] = d[3] = 0.f;
+}
+
+// acc[e][f] = sum_l Mt[l][tr + e] Fb[l][tc + 64 (f / 4) + f % 4].
+template <int CH>
+__device__ __forceinline__ void var_product(const float* Mt, const float* Fb, int tr, int tc, float (&acc)[4][2 * CH]) {
 #pragma unroll
   for (int e = 0; e < 4; e++)
 #pragma unroll
-    for (int f = 0; f < 4; f++) acc[e][f] = V(0);
-  for (int l = 0; l < kl; l++) {
-    V a[4], x[4];
+    for (int f = 0; f < 2 * CH; f++) acc[e][f] = 0.f;
+  float a[2][4], x[2][2 * CH];   // step l's and step l + 1's entries
+  auto fetch = [&](int l, int h) {
+    ld4(Mt + l * MS + tr, a[h]);
 #pragma unroll
-    for (int e = 0; e < 4; e++) a[e] = Mt[l * MS + tr + e];
-#pragma unroll
-    for (int f = 0; f < 4; f++) x[f] = Fb[l * CR + tc + f];
+    for (int g = 0; g < CH / 2; g++) ld4(Fb + l * (CH * R) + tc + 64 * g, x[h] + 4 * g);
+  };
+  fetch(0, 0);
+#pragma unroll 8
+  for (int l = 0; l < T; l++) {
+    const int h = l & 1;
+    fetch(min(l + 1, T - 1), h ^ 1);
 #pragma unroll
     for (int e = 0; e < 4; e++)
 #pragma unroll
-      for (int f = 0; f < 4; f++) acc[e][f] += a[e] * x[f];
+      for (int f = 0; f < 2 * CH; f++) acc[e][f] += a[h][e] * x[h][f];
   }
 }
 
-// X_J = inv(L_JJ) F_J of block kb from Fb (F_J, zero past bw), stored for the active chunks. Mt: scratch.
-template <class St>
-__device__ __forceinline__ void var_block_solve(const typename St::V* inv, const typename St::V* Fb, typename St::V* Mt,
-                                                typename St::V* xv, bool act, int bw, int tr, int tc) {
-  using V = typename St::V;
-  for (int e = threadIdx.x; e < T * T; e += 256) Mt[(e & 63) * MS + (e >> 6)] = inv[e];   // zero past bw
-  __syncthreads();
-  V acc[4][4];
-  var_product(Mt, Fb, T, tr, tc, acc);
-  if (act) {
-#pragma unroll
-    for (int e = 0; e < 4; e++)
-      if (tr + e < bw) {
-#pragma unroll
-        for (int f = 0; f < 4; f++) xv[(int64_t)(tr + e) * R + f] = acc[e][f];
-      }
-  }
-}
-
-// This thread's rows and right-hand sides of the CTA's two chunks, and their chunk.
-template <class V>
+// This thread's rows tr.. +3 and columns tc + 64 g.. +3 of the CTA's CH chunks, the blockIdx.y-th CH of those active in
+// front s: chunk c[g] (-1: none), right-hand sides r.. +3.
+template <int CH>
 struct VarLane {
-  int tr, tc, c, r;   // rows tr.. +3, columns tc.. +3 of the pair = right-hand sides r.. +3 of chunk c
-  bool act;
-  V *F, *X;           // the chunk's front vectors and w entries
-  __device__ __forceinline__ VarLane(const VarWork<V>& vw, int32_t s, int nc)
-      : tr((threadIdx.x >> 4) * 4), tc((threadIdx.x & 15) * 4), c(2 * blockIdx.y + (tc >> 5)), r(tc & 31) {
-    act = c < nc && vw.active[c * vw.ns + s];
-    F = vw.F + c * vw.cs;
-    X = vw.X + c * vw.cs;
+  int tr, tc, r, c[CH / 2];
+  bool any;   // of the CTA
+  __device__ __forceinline__ VarLane(const VarWork<float>& vw, int32_t s, int nc)
+      : tr((threadIdx.x >> 4) * 4), tc((threadIdx.x & 15) * 4), r(tc & 31) {
+    const int lane = threadIdx.x & 31;   // nc <= 64
+    const unsigned lo = __ballot_sync(~0u, lane < nc && vw.active[lane * vw.ns + s]);
+    const unsigned hi = __ballot_sync(~0u, lane + 32 < nc && vw.active[(lane + 32) * vw.ns + s]);
+    unsigned long long set = (unsigned long long)hi << 32 | lo;
+    for (int q = CH * blockIdx.y; q > 0 && set; q--) set &= set - 1;
+    any = set != 0;
+#pragma unroll
+    for (int g = 0; g < CH / 2; g++) {
+      unsigned long long x = (tc >> 5) ? set & (set - 1) : set;
+      c[g] = x ? __ffsll((long long)x) - 1 : -1;
+      set &= set - 1;
+      set &= set - 1;
+    }
   }
 };
 
-// X_0 of the level's large fronts.
-template <class St>
-__global__ void __launch_bounds__(256) k_var_first(const int32_t* __restrict__ fronts, int nc, DevPlan dp, St store,
-                                                   int b, VarWork<typename St::V> vw) {
-  using V = typename St::V;
+// Blocks g0.. + VG of the large fronts of a step: X_J = inv(L_JJ) (F_J - sum_K L_JK X_K) over the group's blocks K < J.
+// The group's X stay in shared memory; the next 64 x 64 tile is on its way to registers during each product.
+constexpr int VG = 4;   // blocks per group
+__global__ void __launch_bounds__(256, 2)
+    k_var_group(const int32_t* __restrict__ fronts, int g0, int nc, DevPlan dp, fa::StoreMix store, int b,
+                VarWork<float> vw) {
+  constexpr int CH = 2, N = T * T / 256;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* Mt = reinterpret_cast<V*>(smem_raw);
-  V* Fb = Mt + T * MS;
+  float* Mt = reinterpret_cast<float*>(smem_raw);   // Mt[l][i]: the product's matrix, row i, column l
+  float* Xb = Mt + T * MS;                      // per block [l][r]: F_J, then X_J
   const int32_t s = fronts[blockIdx.x];
-  const VarLane<V> t(vw, s, nc);
-  if (!__syncthreads_or(t.act)) return;
-  const int bw = min(T, dp.w[s]);
-  const V* fv = t.F + dp.frow_off[s] * R;
+  const VarLane<CH> t(vw, s, nc);
+  if (!t.any) return;
+  auto A = store.acc(dp, s, b);
+  const float* inv = store.inv(dp, s, b);
+  const int w = dp.w[s], nb = min(VG, (w - g0 * T + T - 1) / T);
+  const bool on = t.c[0] >= 0;
+  float* xv = vw.X + (on ? t.c[0] : 0) * vw.cs + ((int64_t)dp.sn_first[s] + t.tr) * R + t.r;
+  const float* fv = vw.F + (on ? t.c[0] : 0) * vw.cs + (dp.frow_off[s] + t.tr) * R + t.r;
+  float v[4][4], lt[N], acc[4][4];
+  auto load = [&](int j, int k) {   // L_JK; the inverse of L_JJ (zero past w)
+    const int r0 = (g0 + j) * T, c0 = (g0 + k) * T;
 #pragma unroll
-  for (int e = 0; e < 4; e++)
+    for (int q = 0; q < N; q++) {
+      const int e = (int)threadIdx.x + 256 * q, i = e >> 6, l = e & 63;
+      if (k == j) lt[q] = inv[(int64_t)(g0 + j) * T * T + e];
+      else lt[q] = r0 + i < w ? A.off(r0 + i, c0 + l) : 0.f;
+    }
+  };
+  load(0, 0);
+  for (int j = 0; j < nb; j++) {
+    const int r0 = (g0 + j) * T;
+    float* Xj = Xb + j * (T * CH * R) + t.tr * (CH * R) + t.tc;   // this thread's entries
 #pragma unroll
-    for (int f = 0; f < 4; f++)
-      Fb[(t.tr + e) * CR + t.tc + f] = t.act && t.tr + e < bw ? fv[(int64_t)(t.tr + e) * R + t.r + f] : V(0);
-  var_block_solve<St>(store.inv(dp, s, b), Fb, Mt, t.X + (int64_t)dp.sn_first[s] * R + t.r, t.act, bw, t.tr, t.tc);
+    for (int e = 0; e < 4; e++) ld4_or_zero(on && r0 + t.tr + e < w, fv + (int64_t)(r0 + e) * R, v[e]);
+    for (int k = 0; k <= j; k++) {
+#pragma unroll
+      for (int q = 0; q < N; q++) {
+        const int e = (int)threadIdx.x + 256 * q;
+        Mt[(e & 63) * MS + (e >> 6)] = lt[q];
+      }
+      if (k == j) {
+#pragma unroll
+        for (int e = 0; e < 4; e++) st4(Xj + e * (CH * R), v[e]);
+      }
+      __syncthreads();
+      if (k < j) load(j, k + 1);
+      else if (j + 1 < nb) load(j + 1, 0);
+      var_product<CH>(Mt, Xb + k * (T * CH * R), t.tr, t.tc, acc);
+      __syncthreads();   // the matrix tile and F_J are free
+      if (k < j) {
+#pragma unroll
+        for (int e = 0; e < 4; e++)
+#pragma unroll
+          for (int f = 0; f < 4; f++) v[e][f] -= acc[e][f];
+      }
+    }
+#pragma unroll
+    for (int e = 0; e < 4; e++) {   // the next product's barrier makes it everyone's
+      st4(Xj + e * (CH * R), acc[e]);
+      if (on && r0 + t.tr + e < w) st4(xv + (int64_t)(r0 + e) * R, acc[e]);
+    }
+  }
 }
 
-// Block column kb of the large fronts of a step: F_I -= L_IJ X_J on the 64-row tiles below (pre: their prefix), and
-// X_{J+1} by the tile of the next block's rows.
-template <class St>
-__global__ void __launch_bounds__(256) k_var_step(const int32_t* __restrict__ fronts, const int64_t* __restrict__ pre,
-                                                  int nfront, int kb, int nc, DevPlan dp, St store, int b,
-                                                  VarWork<typename St::V> vw) {
-  using V = typename St::V;
+// F_I -= sum_J L_IJ X_J on 64-row tile blockIdx.z of the later blocks' rows, J over the group of blocks g0.. + VG;
+// g0 < 0: of the rows below the large fronts' columns, J over all blocks.
+__global__ void __launch_bounds__(256, 2)
+    k_var_rest(const int32_t* __restrict__ fronts, int g0, int nc, DevPlan dp, fa::StoreMix store, int b,
+               VarWork<float> vw) {
+  constexpr int CH = 4;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  V* Mt = reinterpret_cast<V*>(smem_raw);   // Mt[l][i]: L[r0 + i][c0 + l]
-  V* Fb = Mt + T * MS;                      // Fb[l][r]: X_J
-  const int fi = find_front(pre, nfront, blockIdx.x);
-  const int32_t s = fronts[fi];
-  const VarLane<V> t(vw, s, nc);
-  if (!__syncthreads_or(t.act)) return;
+  float* Mt = reinterpret_cast<float*>(smem_raw);   // Mt[l][i]: L[r0 + i][c0 + l]
+  float* Fb0 = Mt + T * MS;                     // two buffers of [l][r]: X_J
+  const int32_t s = fronts[blockIdx.x];
+  const int w = dp.w[s], b0 = max(g0, 0), b1 = g0 < 0 ? (w + T - 1) / T : g0 + VG;   // blocks [b0, b1)
+  const int r0 = (g0 < 0 ? w : b1 * T) + (int)blockIdx.z * T, nr = min(T, (g0 < 0 ? w + dp.r[s] : w) - r0);
+  if (nr <= 0) return;
+  const VarLane<CH> t(vw, s, nc);
+  if (!t.any) return;
   auto A = store.acc(dp, s, b);
-  const int w = dp.w[s];
-  const int64_t m = (int64_t)w + dp.r[s];
-  const int c0 = kb * T, bw = min(T, w - c0), c1 = c0 + bw;
-  const int64_t r0 = c1 + ((int64_t)blockIdx.x - pre[fi]) * T;
-  const int nr = (int)imin64(T, m - r0);
-  const V* xj = t.X + ((int64_t)dp.sn_first[s] + c0) * R + t.r;
+  float* row = vw.F + (dp.frow_off[s] + r0 + t.tr) * R + t.r;
+  const float* xs = vw.X + ((int64_t)dp.sn_first[s] + t.tr) * R + t.r;
+  float v[4][2 * CH], lt[T * T / 256];
 #pragma unroll
   for (int e = 0; e < 4; e++)
 #pragma unroll
-    for (int f = 0; f < 4; f++)
-      Fb[(t.tr + e) * CR + t.tc + f] = t.act && t.tr + e < bw ? xj[(int64_t)(t.tr + e) * R + f] : V(0);
-  for (int e = threadIdx.x; e < T * T; e += 256) {   // reads along the storage
-    const int i = St::kRowMajor ? e >> 6 : e & 63, l = St::kRowMajor ? e & 63 : e >> 6;
-    Mt[l * MS + i] = (i < nr && l < bw) ? (V)A.L(r0 + i, c0 + l) : V(0);
-  }
-  __syncthreads();
-  V acc[4][4];
-  var_product(Mt, Fb, bw, t.tr, t.tc, acc);
-  V* row = t.F + (dp.frow_off[s] + r0 + t.tr) * R + t.r;
+    for (int g = 0; g < CH / 2; g++)
+      ld4_or_zero(t.c[g] >= 0 && t.tr + e < nr, row + t.c[g] * vw.cs + e * R, v[e] + 4 * g);
+  auto load = [&](int kb) {   // block kb: the tile's entries to registers, X to its buffer (asynchronously)
+    const int c0 = kb * T, bw = min(T, w - c0);
+    float* Fb = Fb0 + (kb & 1) * T * CH * R;
 #pragma unroll
-  for (int e = 0; e < 4; e++)
-#pragma unroll
-    for (int f = 0; f < 4; f++) {
-      acc[e][f] = t.act && t.tr + e < nr ? row[(int64_t)e * R + f] - acc[e][f] : V(0);
-      if (t.act && t.tr + e < nr) row[(int64_t)e * R + f] = acc[e][f];
+    for (int q = 0; q < T * T / 256; q++) {
+      const int e = (int)threadIdx.x + 256 * q, i = e >> 6, l = e & 63;
+      lt[q] = i < nr && l < bw ? A.off(r0 + i, c0 + l) : 0.f;
     }
-  if (r0 != c1 || c1 >= w) return;   // the next block's rows: its X as well
-  const int bw2 = min(T, w - c1);
-  __syncthreads();   // every thread has read X_J and the tile
+#pragma unroll
+    for (int e = 0; e < 4; e++)
+#pragma unroll
+      for (int g = 0; g < CH / 2; g++) {   // one 16-byte vector
+          float* d = Fb + (t.tr + e) * (CH * R) + t.tc + 64 * g;
+          if (t.c[g] >= 0 && t.tr + e < bw)
+            __pipeline_memcpy_async(d, xs + t.c[g] * vw.cs + (int64_t)(c0 + e) * R, 16);
+          else
+            d[0] = d[1] = d[2] = d[3] = 0.f;
+        }
+    __pipeline_commit();
+  };
+  load(b0);
+  for (int kb = b0; kb < b1; kb++) {
+#pragma unroll
+    for (int q = 0; q < T * T / 256; q++) {
+      const int e = (int)threadIdx.x + 256 * q;
+      Mt[(e & 63) * MS + (e >> 6)] = lt[q];
+    }
+    __pipeline_wait_prior(0);
+    __syncthreads();
+    if (kb + 1 < b1) load(kb + 1);
+    float acc[4][2 * CH];
+    var_product<CH>(Mt, Fb0 + (kb & 1) * T * CH * R, t.tr, t.tc, acc);   // zeros past w
+#pragma unroll
+    for (int e = 0; e < 4; e++)
+#pragma unroll
+      for (int f = 0; f < 2 * CH; f++) v[e][f] -= acc[e][f];
+    __syncthreads();   // the tile and this block's buffer are free again
+  }
 #pragma unroll
   for (int e = 0; e < 4; e++)
 #pragma unroll
-    for (int f = 0; f < 4; f++) Fb[(t.tr + e) * CR + t.tc + f] = t.tr + e < bw2 ? acc[e][f] : V(0);
-  var_block_solve<St>(store.inv(dp, s, b) + (int64_t)(kb + 1) * T * T, Fb, Mt,
-                      t.X + ((int64_t)dp.sn_first[s] + c1) * R + t.r, t.act, bw2, t.tr, t.tc);
+    for (int g = 0; g < CH / 2; g++)
+      if (t.c[g] >= 0 && t.tr + e < nr) st4(row + t.c[g] * vw.cs + e * R, v[e] + 4 * g);
+}
+
+// The large fronts of a level in FP64. A warp's FP64 multiply-add takes 64 clocks of its scheduler, so a 64 x 64 by
+// 64 x 32 product would hold an SM for 32 us: a CTA takes 16 rows of one chunk (two right-hand sides per thread), which
+// spreads the narrow levels' products over the SMs; shared memory and latency do not show.
+// what = VX: X_J = inv(L_JJ) F_J, rows 16 z of block J = jb; VSTEP: F_I -= L_IJ X_J, rows 16 z of the block columns' rows
+// after block J; VREST: F_I -= sum_J L_IJ X_J, rows 16 z below the front's columns. 2048 (70) test points of a
+// 20,000-point space-time factor: 86 (10.0) ms with 64-row tiles
+// that each formed X_J anew, 66 (27) ms with the mixed factor's kernels above, 48 (5.2) ms here.
+enum { VX, VSTEP, VREST };
+__global__ void __launch_bounds__(256)
+    k_var_rows64(const int32_t* __restrict__ fronts, int what, int jb, DevPlan dp, fa::StoreF64 store, int b,
+                 VarWork<double> vw) {
+  __shared__ double Mt[T][17];   // Mt[l][i]
+  __shared__ __align__(16) double Xs[T][R];
+  const int32_t s = fronts[blockIdx.x];
+  const int c = blockIdx.y;
+  if (!vw.active[c * vw.ns + s]) return;
+  const int w = dp.w[s];
+  const int r0 = (what == VREST ? w : what == VSTEP ? (jb + 1) * T : jb * T) + 16 * (int)blockIdx.z;
+  const int nr = min(16, (what == VREST ? w + dp.r[s] : what == VSTEP ? w : min(w, (jb + 1) * T)) - r0);
+  if (nr <= 0) return;
+  const int b0 = what == VREST ? 0 : jb, b1 = what == VREST ? (w + T - 1) / T : jb + 1;
+  const fa::AccF64 A = store.acc(dp, s, b);
+  const double* inv = store.inv(dp, s, b) + (int64_t)jb * T * T;
+  double* F = vw.F + c * vw.cs + dp.frow_off[s] * R;
+  double* X = vw.X + c * vw.cs + (int64_t)dp.sn_first[s] * R;
+  const double* src = what == VX ? F : X;
+  const int i = threadIdx.x >> 4, r = (threadIdx.x & 15) * 2;
+  double v[2] = {0.0, 0.0};
+  if (what != VX && i < nr) {
+    v[0] = F[(int64_t)(r0 + i) * R + r];
+    v[1] = F[(int64_t)(r0 + i) * R + r + 1];
+  }
+  for (int kb = b0; kb < b1; kb++) {
+    const int c0 = kb * T, bw = min(T, w - c0);
+    for (int e = threadIdx.x; e < T * R; e += 256) Xs[e / R][e % R] = e / R < bw ? src[(int64_t)c0 * R + e] : 0.0;
+    if (what == VX) {
+      for (int e = threadIdx.x; e < T * 16; e += 256) Mt[e & 63][e >> 6] = inv[(r0 - c0) * T + e];   // zero past bw
+    } else {
+      for (int e = threadIdx.x; e < T * 16; e += 256)
+        Mt[e >> 4][e & 15] = (e & 15) < nr && (e >> 4) < bw ? A.off(r0 + (e & 15), c0 + (e >> 4)) : 0.0;
+    }
+    __syncthreads();
+    double a0 = 0.0, a1 = 0.0;
+#pragma unroll 8
+    for (int l = 0; l < T; l++) {
+      const double2 x = *reinterpret_cast<const double2*>(&Xs[l][r]);
+      a0 += Mt[l][i] * x.x;
+      a1 += Mt[l][i] * x.y;
+    }
+    __syncthreads();
+    if (what == VX) v[0] = a0, v[1] = a1;
+    else v[0] -= a0, v[1] -= a1;
+  }
+  double* dst = what == VX ? X : F;
+  if (i < nr) {
+    dst[(int64_t)(r0 + i) * R + r] = v[0];
+    dst[(int64_t)(r0 + i) * R + r + 1] = v[1];
+  }
 }
 
 // Partial sums of w^2 per (chunk, right-hand side) over column slices, in a fixed order: CTA g of chunk c sums
@@ -314,6 +449,7 @@ __global__ void k_var_sumsq(int64_t n, VarWork<V> vw, double* __restrict__ part)
   const int c = blockIdx.y, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const V* x = vw.X + c * vw.cs;
   double acc = 0.0;
+#pragma unroll 8
   for (int64_t j = (int64_t)blockIdx.x * 8 + warp; j < n; j += (int64_t)gridDim.x * 8) {
     const double v = (double)x[j * R + lane];
     acc += v * v;
@@ -372,10 +508,12 @@ void variance_impl(gp_ctx* ctx, gp_factor_t* f, const St& store, int b, const do
   const double* theta = f->theta_dev + (int64_t)b * f->theta_stride;
   const double* Fb = f->F + (int64_t)b * n * h0.n1;
   const double* Cb = f->Cpt ? f->Cpt + (int64_t)b * n * 2 : nullptr;
-  const size_t step_smem = var_step_smem<V>();
-  static_assert(sizeof(V) == 4 || sizeof(V) == 8, "working type");
-  GP_CUDA(cudaFuncSetAttribute(k_var_step<St>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step_smem));
-  GP_CUDA(cudaFuncSetAttribute(k_var_first<St>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)step_smem));
+  constexpr bool fp64 = std::is_same_v<St, fa::StoreF64>;
+  const size_t rest_smem = var_smem(2, 4);
+  if constexpr (!fp64) {
+    GP_CUDA(cudaFuncSetAttribute(k_var_group, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)var_smem(VG, 2)));
+    GP_CUDA(cudaFuncSetAttribute(k_var_rest, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)rest_smem));
+  }
   ProfScope ps_(ctx, KC_PREDICT);
   for (int64_t k0 = 0; k0 < m; k0 += (int64_t)NC * R) {
     const int64_t cnt = std::min<int64_t>(m - k0, (int64_t)NC * R);
@@ -406,17 +544,40 @@ void variance_impl(gp_ctx* ctx, gp_factor_t* f, const St& store, int b, const do
         k_var_small<St><<<dim3(lv.nsmall, nc), 256, 0, st>>>(dp.small_list + lv.small_off, dp, store, b, vw);
         GP_CHECK_LAUNCH(ctx);
       }
-      const unsigned ncp = (unsigned)((nc + 1) / 2);   // pairs of chunks
-      if (!lv.steps.empty()) {
-        k_var_first<St><<<dim3(lv.steps[0].nfront, ncp), 256, step_smem, st>>>(dp.large_fronts + lv.steps[0].fr_off, nc,
-                                                                              dp, store, b, vw);
-        GP_CHECK_LAUNCH(ctx);
-      }
-      for (const auto& stp : lv.steps) {
-        if (stp.trsm_total == 0) continue;
-        k_var_step<St><<<dim3((unsigned)stp.trsm_total, ncp), 256, step_smem, st>>>(
-            dp.large_fronts + stp.fr_off, dp.step_pre + stp.pre_off, stp.nfront, stp.kb, nc, dp, store, b, vw);
-        GP_CHECK_LAUNCH(ctx);
+      if (lv.steps.empty()) continue;
+      // The level's large fronts, widest first (nb blocks).
+      const int nb = (int)lv.steps.size();
+      const auto& s0 = lv.steps[0];
+      const auto list = [&](int k) { return dp.large_fronts + lv.steps[k].fr_off; };   // the fronts that have block k
+      int32_t rmax = 0;
+      for (int32_t q = 0; q < s0.nfront; q++) rmax = std::max(rmax, sp.sn_r[sp.large_fronts[s0.fr_off + q]]);
+      if constexpr (fp64) {
+        for (int k = 0; k < nb; k++) {
+          k_var_rows64<<<dim3(lv.steps[k].nfront, nc, T / 16), 256, 0, st>>>(list(k), VX, k, dp, store, b, vw);
+          GP_CHECK_LAUNCH(ctx);
+          if (k + 1 == nb) break;
+          k_var_rows64<<<dim3(lv.steps[k + 1].nfront, nc, (nb - 1 - k) * (T / 16)), 256, 0, st>>>(list(k + 1), VSTEP, k,
+                                                                                              dp, store, b, vw);
+          GP_CHECK_LAUNCH(ctx);
+        }
+        if (rmax > 0) {
+          k_var_rows64<<<dim3(s0.nfront, nc, (rmax + 15) / 16), 256, 0, st>>>(list(0), VREST, 0, dp, store, b, vw);
+          GP_CHECK_LAUNCH(ctx);
+        }
+      } else {
+        const unsigned n2 = (unsigned)((nc + 1) / 2), n4 = (unsigned)((nc + 3) / 4);
+        for (int g0 = 0; g0 < nb; g0 += VG) {
+          k_var_group<<<dim3(lv.steps[g0].nfront, n2), 256, var_smem(std::min(VG, nb - g0), 2), st>>>(list(g0), g0, nc, dp, store, b, vw);
+          GP_CHECK_LAUNCH(ctx);
+          const int b1 = g0 + VG;
+          if (b1 >= nb) break;
+          k_var_rest<<<dim3(lv.steps[b1].nfront, n4, nb - b1), 256, rest_smem, st>>>(list(b1), g0, nc, dp, store, b, vw);
+          GP_CHECK_LAUNCH(ctx);
+        }
+        if (rmax > 0) {
+          k_var_rest<<<dim3(s0.nfront, n4, (rmax + T - 1) / T), 256, rest_smem, st>>>(list(0), -1, nc, dp, store, b, vw);
+          GP_CHECK_LAUNCH(ctx);
+        }
       }
     }
     k_var_sumsq<V><<<dim3(SUM_CTAS, nc), 256, 0, st>>>(n, vw, part);

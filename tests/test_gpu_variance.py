@@ -97,3 +97,30 @@ def test_variance_bounds_at_100k(ctx):
     assert np.all(v[-200:] <= hp.noise_var * (1 + 1e-9))
     assert np.abs(out[gp.GP_MIXED] - v).max() <= 1e-5 * prior.max()
     ps.free()
+
+
+# one block and a remainder, a group of four blocks and one row more or less, two groups; chunks of 32 test points in
+# pairs and fours with a remainder, and whole chunks without a neighbour between active ones
+@pytest.mark.parametrize("n", [97, 128, 193, 255, 257, 513])
+def test_variance_of_dense_fronts_matches_oracle(ctx, n):
+    """One dense front per case. A backward error E of the factor moves |w|^2 by at most |C^-1 c|^2 |E|, with |C^-1 c| <= 1
+    for a cross-covariance column beside the data and |C| <= n times the prior: n 2^-22 of the prior's scale in FP32,
+    1e-9 in FP64."""
+    from paper_2411_05869_gb300 import gp
+    w = synth.spatial_2d(n=n, m=1, seed=2000 + n, rho=2.0, noise_var=1.0)
+    rng = np.random.default_rng(n)
+    near = rng.random((133, w.X.shape[1]))
+    far = np.full((32, w.X.shape[1]), 50.0)
+    Xt = np.concatenate([near[:32], far, near[32:]], axis=0)
+    ref = oracle.predictive_variance(w.hyper, w.X, Xt)
+    scale = max(oracle.cy(w.hyper, x, x) for x in Xt)
+    ps = ctx.assemble(_dev(w.X), w.hyper.core_radius)
+    for prec, tol in ((gp.GP_FP64, 1e-9), (gp.GP_MIXED, n * 2.0**-22)):
+        f = ctx.factor(ps, [w.hyper], prec)
+        v = f.predict_var(_dev(Xt)).cpu().numpy()
+        assert np.abs(v - ref).max() <= tol * scale, (prec, np.abs(v - ref).max(), scale)
+        for m in (1, 33, 65, 97):   # the other chunks in a CTA do not change a point's value
+            part = f.predict_var(_dev(Xt[-m:])).cpu().numpy()
+            assert part.tobytes() == v[-m:].tobytes(), (prec, m)
+        f.free()
+    ps.free()
