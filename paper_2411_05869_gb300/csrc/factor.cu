@@ -26,6 +26,7 @@
 #include "f64_digits.cuh"
 #include "gp_internal.cuh"
 #include "potrf64.cuh"
+#include "small_front.cuh"
 #include "tc_gemm.cuh"
 
 void values_run(gp_ctx* ctx, gp_factor_t* f);
@@ -56,49 +57,23 @@ __device__ __forceinline__ double* front_at(const FrontRef& fr, int64_t i, int64
   return j < fr.w ? fr.P + j * fr.m + i : fr.Uu + (j - fr.w) * fr.r + (i - fr.w);
 }
 
-__device__ __forceinline__ double checked_sqrt(double d, int32_t* notpd, int32_t col) {
-  if (!(d > 0.0)) {
-    atomicMin(notpd, col);
-    return 1.0;
-  }
-  return sqrt(d);
-}
-
 // Whole partial factorization of a front of order <= GP_SMALL_M in shared memory.
-__global__ void k_small_front(const int32_t* __restrict__ list, DevPlan dp, double* __restrict__ panels,
-                              double* __restrict__ upd, int64_t PE, int64_t UE, int32_t* __restrict__ notpd) {
+__global__ void __launch_bounds__(sf::THREADS)
+    k_small_front(const int32_t* __restrict__ list, DevPlan dp, double* __restrict__ panels, double* __restrict__ upd,
+                  int64_t PE, int64_t UE, int32_t* __restrict__ notpd) {
   extern __shared__ double A[];   // m x m, column-major, lower part used
   int32_t s = list[blockIdx.x];
   int b = blockIdx.y;
   FrontRef fr = front_of(dp, s, panels + (int64_t)b * PE, upd + (int64_t)b * UE);
   const int m = (int)fr.m, w = fr.w;
   const int32_t first = dp.sn_first[s];
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    int i = t % m, j = t / m;
-    if (i >= j) A[t] = *front_at(fr, i, j);
-  }
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // a warp per column: along the storage
+  for (int j = ty; j < m; j += sf::THREADS / 32)
+    for (int i = j + tx; i < m; i += 32) A[j * m + i] = *front_at(fr, i, j);
   __syncthreads();
-  __shared__ double piv;
-  for (int k = 0; k < w; k++) {
-    if (threadIdx.x == 0) {
-      piv = checked_sqrt(A[k * m + k], notpd + b, first + k);
-      A[k * m + k] = piv;
-    }
-    __syncthreads();
-    double inv = 1.0 / piv;
-    for (int i = k + 1 + threadIdx.x; i < m; i += blockDim.x) A[k * m + i] *= inv;
-    __syncthreads();
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // 8 columns x 32 rows (blockDim = 256)
-    for (int j = k + 1 + ty; j < m; j += 8) {
-      const double ajk = A[k * m + j];
-      for (int i = j + tx; i < m; i += 32) A[j * m + i] -= A[k * m + i] * ajk;
-    }
-    __syncthreads();
-  }
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    int i = t % m, j = t / m;
-    if (i >= j) *front_at(fr, i, j) = A[t];
-  }
+  sf::eliminate(A, m, w, first, notpd + b);
+  for (int j = ty; j < m; j += sf::THREADS / 32)
+    for (int i = j + tx; i < m; i += 32) *front_at(fr, i, j) = A[j * m + i];
 }
 
 __device__ __forceinline__ int find_front(const int64_t* pre, int nfront, int64_t t) {
@@ -661,7 +636,7 @@ static void factor_body(gp_ctx* ctx, gp_factor_t* f) {
         mmax = std::max(mmax, sp.sn_w[s] + sp.sn_r[s]);
       }
       ProfScope ps_(ctx, KC_FRONT_SMALL);
-      k_small_front<<<dim3(lv.nsmall, B), 256, (size_t)mmax * mmax * sizeof(double), st>>>(
+      k_small_front<<<dim3(lv.nsmall, B), sf::THREADS, (size_t)mmax * mmax * sizeof(double), st>>>(
           dp.small_list + lv.small_off, dp, f->panels, f->upd, PE, UE, f->notpd);
       GP_CHECK_LAUNCH(ctx);
     }

@@ -25,6 +25,7 @@
 
 #include "extend_add.cuh"
 #include "gp_internal.cuh"
+#include "small_front.cuh"
 #include "tc_gemm.cuh"
 
 void values_run_mixed(gp_ctx* ctx, gp_factor_t* f);
@@ -71,51 +72,24 @@ __device__ __forceinline__ void mix_set(const MixFront& fr, int64_t i, int64_t j
     fr.Uu[(i - fr.w) * fr.r + (j - fr.w)] = (float)v;
   }
 }
-__device__ __forceinline__ double checked_sqrt(double d, int32_t* notpd, int32_t col) {
-  if (!(d > 0.0)) {
-    atomicMin(notpd, col);
-    return 1.0;
-  }
-  return sqrt(d);
-}
 
 // Fronts of order <= GP_SMALL_M: the whole partial factorization in FP64 shared memory.
-__global__ void k_small_front32(const int32_t* __restrict__ list, DevPlan dp, float* __restrict__ p32,
-                                double* __restrict__ dg, float* __restrict__ u32, int64_t P32E, int64_t DE,
-                                int64_t UE, int32_t* __restrict__ notpd) {
+__global__ void __launch_bounds__(sf::THREADS)
+    k_small_front32(const int32_t* __restrict__ list, DevPlan dp, float* __restrict__ p32, double* __restrict__ dg,
+                    float* __restrict__ u32, int64_t P32E, int64_t DE, int64_t UE, int32_t* __restrict__ notpd) {
   extern __shared__ double A[];
   int32_t s = list[blockIdx.x];
   int b = blockIdx.y;
   MixFront fr = mix_front(dp, s, p32 + (int64_t)b * P32E, dg + (int64_t)b * DE, u32 + (int64_t)b * UE);
   const int m = (int)fr.m, w = fr.w;
   const int32_t first = dp.sn_first[s];
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    int i = t % m, j = t / m;
-    if (i >= j) A[t] = mix_get(fr, i, j);
-  }
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;   // a warp per row: along the storage
+  for (int i = ty; i < m; i += sf::THREADS / 32)
+    for (int j = tx; j <= i; j += 32) A[j * m + i] = mix_get(fr, i, j);
   __syncthreads();
-  __shared__ double piv;
-  for (int k = 0; k < w; k++) {
-    if (threadIdx.x == 0) {
-      piv = checked_sqrt(A[k * m + k], notpd + b, first + k);
-      A[k * m + k] = piv;
-    }
-    __syncthreads();
-    double inv = 1.0 / piv;
-    for (int i = k + 1 + threadIdx.x; i < m; i += blockDim.x) A[k * m + i] *= inv;
-    __syncthreads();
-    // trailing lower triangle: 8 columns x 32 rows of threads (blockDim = 256)
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
-    for (int j = k + 1 + ty; j < m; j += 8) {
-      const double ajk = A[k * m + j];
-      for (int i = j + tx; i < m; i += 32) A[j * m + i] -= A[k * m + i] * ajk;
-    }
-    __syncthreads();
-  }
-  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
-    int i = t % m, j = t / m;
-    if (i >= j) mix_set(fr, i, j, A[t]);
-  }
+  sf::eliminate(A, m, w, first, notpd + b);
+  for (int i = ty; i < m; i += sf::THREADS / 32)
+    for (int j = tx; j <= i; j += 32) mix_set(fr, i, j, A[j * m + i]);
 }
 
 __device__ __forceinline__ int find_front(const int64_t* pre, int nfront, int64_t t) {
@@ -1441,7 +1415,7 @@ void factor_run_mixed(gp_ctx* ctx, gp_factor_t* f) {
         mmax = std::max(mmax, sp.sn_w[s] + sp.sn_r[s]);
       }
       ProfScope ps_(ctx, KC_FRONT_SMALL);
-      k_small_front32<<<dim3(lv.nsmall, B), 256, (size_t)mmax * mmax * sizeof(double), st>>>(
+      k_small_front32<<<dim3(lv.nsmall, B), sf::THREADS, (size_t)mmax * mmax * sizeof(double), st>>>(
           dp.small_list + lv.small_off, dp, f->panels32, f->diag, f->upd32, P32E, DE, UE, f->notpd);
       GP_CHECK_LAUNCH(ctx);
     }
