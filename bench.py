@@ -29,9 +29,9 @@ import numpy as np
 ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
-# FP64 FMA throughput of a GB300 of this machine, measured with a dependent-free FP64 FMA loop over all SMs (the FP64
-# path's A7 kernels are bound by it; FP64 tensor-core DMMA measured no faster on this part)
-MEASURED_FP64_TFLOPS = 1.011
+# The FP64 path's updates and TRSMs take an FP64 product as this many FP16 digit products on the tensor cores (an FP64 FMA
+# loop over all SMs measured 1.011 TFLOP/s on a GB300, and FP64 tensor-core DMMA no more).
+FP64_DIGIT_PRODUCTS = 26
 NOMINAL_TF32_OVER_BF16 = 1.1 / 2.25
 
 
@@ -833,8 +833,9 @@ def main():
         peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"]) * NOMINAL_TF32_OVER_BF16
         bound, peak_note = "tensor", f"TF32 = {peak_src} bf16 sustained x nominal 1.1/2.25 (of {peak_src})"
     else:
-        peak = MEASURED_FP64_TFLOPS
-        bound, peak_note = "alu", "FP64 FMA throughput measured on this pool"
+        peak = peaks.get("bf16_tflops_sustained", peaks["bf16_tflops"]) / FP64_DIGIT_PRODUCTS
+        bound, peak_note = "tensor", (f"FP16 = {peak_src} bf16 sustained / {FP64_DIGIT_PRODUCTS} digit products per FP64 "
+                                      f"product (of {peak_src})")
     # the dominant kernel among the classes with a flop count (the tensor-core updates, POTRF, TRSM)
     dom = max(["potrf", "trsm", "update", "update_left"], key=lambda k: prof[k][0])
     d_ms, d_n, d_fl_front = prof[dom]
@@ -938,9 +939,10 @@ def main():
 KERNEL_OF_CLASS_MIXED = {"update": "k_update_ws<256, pair> (group-end updates: 256 x 256 CTA-pair tcgen05 MMAs)",
                          "update_left": "k_update_ws<128> (left-looking updates of block-column pairs, 128 x 128 tiles)",
                          "potrf": "k_potrf_pair (FP32 elimination with inverses) + k_potrf_tiles64 (FP64 L_11)",
-                         "trsm": "k_trsm32_pair", "extend_add": "k_extend_add32"}
-KERNEL_OF_CLASS_FP64 = {"update": "k_update (FP64 trailing updates)", "potrf": "k_potrf", "trsm": "k_trsm",
-                        "extend_add": "k_extend_add"}
+                         "trsm": "k_trsm32_pair", "extend_add": "k_assemble32"}
+KERNEL_OF_CLASS_FP64 = {"update": "k_update64<group> (group-end updates: 26 digit products on the FP16 tensor cores)",
+                        "update_left": "k_update64 (left-looking updates)", "potrf": "k_potrf64", "trsm": "k_trsm64",
+                        "extend_add": "k_assemble64"}
 
 # DRAM bytes per launch of the dominant kernel by (workload, class, update blocking[, operand split]), from ncu
 # captures of the current kernel; None where there is none. FP16 pairs, station_120k: all 79 group-end launches of

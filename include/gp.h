@@ -121,7 +121,9 @@ typedef struct {
  *     launch of that factorization skips its tiles; a solve task goes on with what it has. The factor then
  *     reports GP_ERR_TIMEOUT: gp_factor_info (timed_out = 1) and gp_loglik return it, and the log-likelihoods are
  *     NaN. No legitimate wait comes near the defaults; tiny limits make waits run out on purpose (a test of this
- *     path). The next gp_factor_update of the factor starts clean.
+ *     path). The next gp_factor_update of the factor starts clean. The waits inside a GP_FP64 factorization (its
+ *     tensor-core kernels, and the two CTAs that factor a diagonal tile) always have the default limits; one that runs
+ *     out is reported in the same way.
  *   GP_OPT_REFINE_EXP (default 10, 6..15): gp_loglik's GP_MIXED refinement stops once every proposal's FP64
  *     relative residual |r - C alpha| / |r| is at most 10^-value (or after 10 corrections). Its quadratic form is
  *     second order in that residual, so the log-likelihood does not need more; gp_predict refines alpha to 1e-12
@@ -322,10 +324,10 @@ GP_API gp_status gp_loglik_iterative(gp_ctx* ctx, gp_factor_t* f, int b, const d
  * kernel classes with CUDA events on the context stream; gp_profile(ctx, 0) stops. gp_profile_read
  * synchronises the stream and returns, for one class, the summed device time (ms), the launch count and the
  * useful flops those launches performed (0 where no flop count applies). Classes:
- *   0 A4 kernel values, 1 A7 extend-add (GP_MIXED: with the zeroing of the update matrices), 2 A7 small
+ *   0 A4 kernel values, 1 A7 extend-add (with the zeroing of the update matrices), 2 A7 small
  *   fronts, 3 A7 diagonal-block POTRF, 4 A7 TRSM, 5 A7 trailing update (SYRK/GEMM; with GP_MIXED the
  *   group-end updates), 6 A8-A10 solve sweep (one span per gp_loglik), 7 A12 prediction, 8 A1-A6 assembly,
- *   9 A7 left-looking block-column updates (GP_MIXED).
+ *   9 A7 left-looking block-column updates.
  * Errors: GP_ERR_ARG (class out of range), GP_ERR_CUDA. */
 GP_API gp_status gp_profile(gp_ctx* ctx, int enable);
 GP_API gp_status gp_profile_read(gp_ctx* ctx, int kclass, double* total_ms, int64_t* launches, double* flops);

@@ -111,7 +111,8 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(p64::THREADS, 1)
   tcg::cluster_sync();   // no CTA leaves while the other may write into it
 }
 
-// rho of every row of L (permuted order): sqrt(C_jj) <= 2^(rho + 1), from the exponent of the assembled diagonal; |L_ji| <= sqrt(C_jj) makes it a scale for the digits of the whole row.
+// rho of every row of L (permuted order): sqrt(C_jj) <= 2^(rho + 1), from the exponent of the assembled diagonal;
+// |L_ji| <= sqrt(C_jj) makes it a scale for the digits of the whole row.
 __global__ void __launch_bounds__(256) k_row_scale(DevPlan dp, int64_t n, const double* __restrict__ panels, int64_t PE,
                                                    int32_t* __restrict__ rho) {
   const int b = blockIdx.y;
