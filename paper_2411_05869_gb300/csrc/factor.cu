@@ -254,7 +254,7 @@ __global__ void __launch_bounds__(256, 1)
     tcg::mma_commit(&bar);
   }
   __syncwarp();
-  bool ok = skip || tcg::mbar_wait(&bar, 0, lim);
+  bool ok = skip || tcg::mbar_wait_warp(&bar, 0, lim);
   if (!ok) {   // record it, then wait for the MMAs issued before tensor memory is given back
     atomicExch(err, 1);
     tcg::mbar_wait(&bar, 0);
@@ -486,7 +486,7 @@ __global__ void __launch_bounds__(U64_THREADS, 1)
   } else {   // epilogue: warp reads TMEM lanes 32 (warp % 4) .. + 31, columns [32 h, 32 h + 32) of each level
     const int q = warp & 3, h = (warp - 2) >> 2;
     uint32_t aph = 0;
-    for (int64_t tt = blockIdx.x; tt < ntiles && !*abort_flag; tt += gridDim.x) {
+    for (int64_t tt = blockIdx.x; tt < ntiles && !__any_sync(0xffffffffu, *abort_flag); tt += gridDim.x) {
       const Tile64 u = decode_tile64<GROUP>(fronts, pre, nfront, total, kb, dp, slot_of, tt);
       double* P = panels + (int64_t)u.b * PE + dp.loff[u.s];
       double* U = upd + (int64_t)u.b * UE + dp.uoff[u.s];
@@ -509,11 +509,10 @@ __global__ void __launch_bounds__(U64_THREADS, 1)
       const int nv = i < u.m ? (int)imin64(32, imin64(i + 1, u.jlim) - jb) : 0;   // this row's entries: the first nv columns
       double* p = colp(jb) + i;   // dereferenced only below nv
       int wl = (int)imin64(64, u.w - jb);   // columns from wl on lie in the update matrix
-      if (!tcg::mbar_wait(tfull, aph, lim)) {
+      if (!tcg::mbar_wait_warp(tfull, aph, lim)) {
         fail();
         break;
       }
-      __syncwarp();
       tcg::tc_fence_after();
 #pragma unroll 1
       for (int g = 0; g < 4; g++) {

@@ -896,7 +896,7 @@ __global__ void __launch_bounds__(UW_THREADS, 1)
     const int q = warp & 3, h = (warp - 2) >> 2;
     float* slab = epi + (warp - 2) * 1024;
     uint32_t acc = 0, aph = 0;
-    for (int64_t tt = t_first; tt < ntiles && !*abort_flag; tt += t_step) {
+    for (int64_t tt = t_first; tt < ntiles && !__any_sync(0xffffffffu, *abort_flag); tt += t_step) {
       const UTile u = decode_tile<TN, PAIR>(fronts, pre, nfront, total, kb, mode, group, dp, slot_of, tt, rank);
       float* P = p32 + (int64_t)u.b * P32E + dp.loff32[u.s];
       float* U = u32 + (int64_t)u.b * UE + dp.uoff[u.s];
@@ -919,7 +919,7 @@ __global__ void __launch_bounds__(UW_THREADS, 1)
           }
         }
       }
-      if (!tcg::mbar_wait(&tfull[acc], aph, lim)) {
+      if (!tcg::mbar_wait_warp(&tfull[acc], aph, lim)) {
         fail();
         break;
       }

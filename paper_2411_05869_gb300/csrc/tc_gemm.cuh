@@ -58,6 +58,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, WaitLi
   }
   return false;
 }
+// A converged warp's wait: one answer for all its lanes, true if any of them saw the phase complete, so that the warp stays
+// together for the aligned tensor-memory instructions that follow (lanes that gave up on their own would leave the others
+// in them).
+__device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, WaitLimit lim = DEFAULT_WAIT) {
+  const bool ok = __any_sync(0xffffffffu, mbar_wait(bar, parity, lim));
+  __syncwarp();
+  return ok;
+}
 // The same, acquiring at cluster scope (for arrivals from another CTA of the cluster).
 __device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity, WaitLimit lim = DEFAULT_WAIT) {
   const uint64_t t0 = global_ns();
