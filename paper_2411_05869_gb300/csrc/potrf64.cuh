@@ -15,8 +15,10 @@
 // error 2^-60 of the rows' scales: smaller than the rounding of FP64 (2^-53 of a_ii on a_ii >= 2^-4). 1 / sqrt(pivot)
 // comes from the FP32 approximation by one cubic step in 64-bit integers.
 // The inverse: forward elimination of the identity, R_i -= l_ik X_k, X_k = R_k / l_kk, in the same halves, every row with
-// an exponent of its own: its terms are kept at 2^-3 of the row's scale, so that the 63 of them cannot overflow 64 bits,
-// and a row whose next term is larger is shifted first (at 2^-5 the solves' residuals came out 1.5 times larger).
+// an exponent of its own: its terms are kept at 2^-3 of the row's scale, so that the 63 of them in H cannot overflow 64
+// bits, and a row whose next term is larger is shifted first (at 2^-5 the solves' residuals came out 1.5 times larger).
+// The cross terms of C are below 2^59 + 2^56 each (the low half of l is not bounded by the shift), so C's whole units of
+// 2^-60 are added to H after every eight columns: low halves that all have one sign would otherwise wrap it.
 // A step is a chain of dependent instructions (pivot, reciprocal root, scaling, one hand-over), so nothing else waits
 // for anything: every column of the factor and row of the inverse has a place and an mbarrier of its own, and the warp
 // that holds the next one updates and publishes it before it does the rest of its updates.
@@ -434,6 +436,15 @@ __device__ __forceinline__ void inverse(Smem& sm, double* __restrict__ DI, uint8
         mad(C[r][1], lr[r].y, x1.x);
       }
     }
+    if ((k & 7) == 7) {   // the cross sums' whole units go over
+#pragma unroll
+      for (int r = 0; r < 8; r++)
+#pragma unroll
+        for (int c = 0; c < 2; c++) {
+          H[r][c] += C[r][c] >> 30;
+          C[r][c] &= (1LL << 30) - 1;
+        }
+    }
   }
   // rows past the tile's width: zero
   for (int i = bw + w; i < PT; i += 8) {
@@ -449,4 +460,30 @@ __device__ __forceinline__ void inverse(Smem& sm, double* __restrict__ DI, uint8
 }
 
 }  // namespace p64
+
+// POTRF of the diagonal tile of block column kb, its inverse in FP64 (row-major, for the solves) and the inverse's digit
+// planes for the step's TRSM, a cluster of two CTAs per large front.
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(p64::THREADS, 1)
+    k_potrf64(const int32_t* __restrict__ fronts, int kb, DevPlan dp, double* __restrict__ panels, int64_t PE,
+              int32_t* __restrict__ notpd, double* __restrict__ dinv, int64_t DE, uint8_t* __restrict__ itile,
+              int64_t IE, int32_t* __restrict__ err) {
+  extern __shared__ __align__(16) uint8_t potrf_raw[];
+  p64::Smem& sm = *reinterpret_cast<p64::Smem*>(potrf_raw);
+  const int fi = blockIdx.x >> 1;
+  const int32_t s = fronts[fi];
+  const int b = blockIdx.y;
+  const int w = dp.w[s];
+  const int64_t m = (int64_t)w + dp.r[s];
+  const int c0 = kb * p64::PT, bw = min(p64::PT, w - c0);
+  const int32_t first = dp.sn_first[s] + c0;
+  double* P = panels + (int64_t)b * PE + dp.loff[s] + (int64_t)c0 * m + c0;
+  if (threadIdx.x < 3 * p64::PT) tcg::mbar_init(&sm.lready[threadIdx.x], 1);   // the three arrays
+  asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+  tcg::cluster_sync();
+  if (tcg::cluster_ctarank() == 0) p64::factor(sm, P, m, bw, first, notpd + b, err);
+  else p64::inverse(sm, dinv + (int64_t)b * DE + dp.doff[s] + (int64_t)kb * p64::PT * p64::PT,
+                    itile + (int64_t)b * IE + (int64_t)fi * p64::TILE_BYTES, bw, err);
+  tcg::cluster_sync();   // no CTA leaves while the other may write into it
+}
+
 }  // namespace
