@@ -113,17 +113,17 @@ typedef struct {
  *     log-determinant is summed in FP64 from their diagonals; FP32 is faster on GB300 (its FP64 pipe is slow) at
  *     the cost of an FP32-accurate diagonal of L in the log-determinant.
  *   GP_OPT_WAIT_POLLS (default 2^26, 1..2^32-1) and GP_OPT_WAIT_NS (default 1e9, >= 0): the limits of every
- *     bounded wait of the GP_MIXED tensor-core kernels (an mbarrier phase awaited by one warp role from another:
- *     operand copies landed, MMAs done, accumulator drained) and of the solves' tasks in both precisions (a task
- *     awaiting a block another task of the same launch publishes). A wait that runs out after that many polls or
- *     nanoseconds records the failure in the factor and ends its wait: a tensor-core kernel winds down (after
- *     waiting, with the default limits, for the copies and MMAs it already issued) and every later tensor-core
- *     launch of that factorization skips its tiles; a solve task goes on with what it has. The factor then
- *     reports GP_ERR_TIMEOUT: gp_factor_info (timed_out = 1) and gp_loglik return it, and the log-likelihoods are
- *     NaN. No legitimate wait comes near the defaults; tiny limits make waits run out on purpose (a test of this
- *     path). The next gp_factor_update of the factor starts clean. The waits inside a GP_FP64 factorization (its
- *     tensor-core kernels, and the two CTAs that factor a diagonal tile) always have the default limits; one that runs
- *     out is reported in the same way.
+ *     bounded wait of the factorizations' tensor-core kernels in both precisions (an mbarrier phase awaited by one
+ *     warp role from another: operand copies landed, MMAs done, accumulator drained) and of the solves' tasks in
+ *     both precisions (a task awaiting a block another task of the same launch publishes). The waits between the two
+ *     CTAs that factor a GP_FP64 diagonal tile always have the default limits. A wait that runs out after that many
+ *     polls or nanoseconds records the failure in the factor and ends its wait: a tensor-core kernel winds down
+ *     (after waiting, with the default limits, for the copies and MMAs it already issued) and every later
+ *     tensor-core launch of that factorization skips its tiles; a diagonal tile or a solve task goes on with what it
+ *     has. The factor then reports GP_ERR_TIMEOUT: gp_factor_info returns it (timed_out = 1), and so does gp_loglik
+ *     where it waits for the GPU (GP_MIXED on the legacy default stream); the log-likelihoods are NaN. No legitimate
+ *     wait comes near the defaults; tiny limits make waits run out on purpose (a test of this path). The next
+ *     gp_factor_update of the factor starts clean, with the limits that the factor was made with.
  *   GP_OPT_REFINE_EXP (default 10, 6..15): gp_loglik's GP_MIXED refinement stops once every proposal's FP64
  *     relative residual |r - C alpha| / |r| is at most 10^-value (or after 10 corrections). Its quadratic form is
  *     second order in that residual, so the log-likelihood does not need more; gp_predict refines alpha to 1e-12

@@ -101,7 +101,7 @@ struct gp_ctx {
   // options (gp_set_option); they apply to factors created afterwards
   int opt_diag_fp32 = 0;     // GP_MIXED: diagonal blocks factored in FP32
   int opt_split_f16 = 1;     // GP_MIXED: FP16 operand pairs for the tensor-core updates (0: TF32 pairs)
-  tcg::WaitLimit opt_wait = tcg::DEFAULT_WAIT;   // GP_MIXED: limits of the tensor-core kernels' bounded waits
+  tcg::WaitLimit opt_wait = tcg::DEFAULT_WAIT;   // limits of the bounded waits (tensor-core kernels, solve tasks)
   int opt_refine_exp = 10;   // GP_MIXED: gp_loglik's refinement stops at |r - C alpha| / |r| <= 10^-opt_refine_exp
   ~gp_ctx() {
     if (ev_fork) cudaEventDestroy(ev_fork);
