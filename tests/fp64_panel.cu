@@ -26,7 +26,7 @@ struct Buffers {   // frees what it allocated
 
 // panel: in the covariance, out L. dinv: 64 x 64, the inverse of the diagonal block, row-major. diag: the m rows' variances.
 // status[0]: smallest failing column (INT32_MAX: none), status[1]: nonzero if a wait ran out. Returns a cudaError_t.
-extern "C" int fp64_panel(double* panel, int m, int bw, const double* diag, double* dinv, int32_t* status) {
+extern "C" __attribute__((visibility("default"))) int fp64_panel(double* panel, int m, int bw, const double* diag, double* dinv, int32_t* status) {
   if (m < 1 || m > 4096 || bw < 1 || bw > 64 || bw > m) return -1;
   const int nt = (m - bw + TRSM_ROWS - 1) / TRSM_ROWS;
   std::vector<int32_t> rows(m), rho(m);
