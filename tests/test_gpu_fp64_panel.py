@@ -44,16 +44,19 @@ def panel(tmp_path_factory):
     return run
 
 
-@pytest.mark.parametrize("v", [0.75 * 2.0 ** -33, 0.99 * 2.0 ** -33, 0.75 * 2.0 ** -32, 0.99 * 2.0 ** -32, 0.99 * 2.0 ** -31])
-@pytest.mark.parametrize("a", [0.9375, 1.0])
-def test_inverse_whose_low_halves_have_one_sign(panel, a, v):
-    """L = I but for the column -a and the row v, entries whose low 30 bits are all near the largest: the inverse's cross
-    sums add up 62 terms of one sign. The inverse is good to 2^-57 of each row's largest entry (its rows are cut at 2^-60 and
-    come from at most 63 products), whose rows are at most 63 long against L's of at most 2: 2^-50 in the product."""
-    L = np.eye(64)
+@pytest.mark.parametrize("terms", [8, 15, 17, 33, 62])
+@pytest.mark.parametrize("low", [0.99, -0.99, 0.6])
+def test_inverse_whose_low_halves_have_one_sign(panel, low, terms):
+    """Rows 1..62 of the inverse start with nearly the largest entry a row can have, and row 63 of L holds low 2^29 units of
+    2^-60 (once at the scale of its row) in the first `terms` of them: all its cross products have one sign and add up to
+    terms low 2^59. The inverse is good to 2^-57 of each row's largest entry (cut at 2^-60, from at most 63 products):
+    2^-50 of it in a product with rows of L that are at most 2 long."""
+    a, d, v = 255 / 128, 1027 / 8192, low * 2.0 ** -35   # exact squares: L L^T is exact but for its last diagonal entry
+    L = np.diag(np.r_[1.0, np.full(62, d), 1.0])
     L[1:63, 0] = -a
-    L[63, 1:63] = v
+    L[63, 1:terms + 1] = v
     A = np.tril(L @ L.T)
     P, D, bad = panel(A, np.diag(A))
     assert bad is None
-    assert np.abs(D @ P - np.eye(64)).max() <= 2.0 ** -50
+    E = np.abs(D.astype(np.longdouble) @ P.astype(np.longdouble) - np.eye(64))
+    assert (E <= 2.0 ** -49 * np.abs(D).max(1, keepdims=True)).all(), float(E.max())
