@@ -112,24 +112,30 @@ __device__ __forceinline__ int64_t to_biased(const Norm& r, int rho) {
 __device__ __forceinline__ double fix2double(int64_t v, int e) { return to_double(normalise(v, e + 62)); }   // v 2^e
 
 // The levels' sums (level l weighs 2^(-18 - 9 l) of the product of the two scales, 2^e) as one number.
-__device__ __forceinline__ int64_t high_levels(const float (&a)[NL]) {   // levels 0..3 in units of 2^-45
-  int64_t t = (int64_t)__float2int_rn(a[0]) * (1 << 27);
-  t += (int64_t)__float2int_rn(a[1]) * (1 << 18);
-  t += (int64_t)__float2int_rn(a[2]) * (1 << 9);
-  return t + (int64_t)__float2int_rn(a[3]);
+__device__ __forceinline__ int64_t high_levels(float a0, float a1, float a2, float a3) {   // levels 0..3 in units of 2^-45
+  int64_t t = (int64_t)__float2int_rn(a0) * (1 << 27);
+  t += (int64_t)__float2int_rn(a1) * (1 << 18);
+  t += (int64_t)__float2int_rn(a2) * (1 << 9);
+  return t + (int64_t)__float2int_rn(a3);
 }
 // The dot product of two rows of a Cholesky factor (at most 4): units of 2^-59. Levels 4 to 6 are added in FP32 before
 // the conversion (at most 2^30 units, and the sum's rounding matters only where the diagonal's squares make it large).
+// A row that is longer than its variance allows (it is not a row of a Cholesky factor: no positive definite covariance)
+// must not wrap: level 0 is held at twice its bound (8, and the other levels add or take less than 2), so that the row's
+// diagonal comes out below zero.
 __device__ __forceinline__ Norm product_rows(const float (&a)[NL], int e) {
   const float low = fmaf(a[6], 0x1p-13f, fmaf(a[5], 0x1p-4f, a[4] * 0x1p5f));
-  return normalise(high_levels(a) * (1LL << 14) + (int64_t)__float2int_rn(low), e + 3);
+  const float a0 = fminf(fmaxf(a[0], -0x1p21f), 0x1p21f);
+  return normalise(high_levels(a0, a[1], a[2], a[3]) * (1LL << 14) + (int64_t)__float2int_rn(low), e + 3);
 }
 // A dot product of 64 terms of at most 1 that the caller knows to be at most 2^eb: units of 2^(eb - 61) where the levels
-// give that much, 2^-55 of the scales at the coarsest (the 64 terms' bound), 2^-69 at the finest.
-__device__ __forceinline__ Norm product_any(const float (&a)[NL], int e, int eb) {
+// give that much, 2^-55 of the scales at the coarsest (the 64 terms' bound), 2^-69 at the finest. Sets `over` where it is
+// more than 1.5 times 2^eb (levels 0 and 1 tell, to 2^-12); the result is then any number.
+__device__ __forceinline__ Norm product_any(const float (&a)[NL], int e, int eb, bool& over) {
   const int S = 16 - max(min(eb - e, 6), -8);   // extra bits below the levels 0..3
   const float low = fmaf(a[6], 0x1p-27f, a[5] * 0x1p-18f) * __int_as_float((127 + S) << 23);
-  int64_t v = high_levels(a) << S;
+  over = over || fabsf(fmaf(a[1], 0x1p-9f, a[0])) > 1.5f * __int_as_float((127 + 34 - S) << 23);
+  int64_t v = high_levels(a[0], a[1], a[2], a[3]) << S;
   v += (int64_t)__float2int_rn(a[4]) * (int64_t)(1 << (S - 9));
   return normalise(v + (int64_t)__float2int_rn(low), e + 17 - S);
 }

@@ -13,8 +13,10 @@
 //      times the inverse, and at a group's end the rows and columns after it receive the group's updates at once
 //      (K = 256). The products of the last three run on the FP16 tensor cores, on six 9-bit digits per FP64 entry
 //      (f64_digits.cuh), since GB300's FP64 pipe gives 1 TFLOP/s.
-// A non-positive pivot records the smallest failing permuted column of that proposal and continues with a
-// unit pivot, so the launch sequence is fixed and no kernel traps.
+// A non-positive pivot records the smallest failing permuted column of that proposal and the factorization continues
+// (small fronts with a unit pivot, diagonal tiles of large fronts with any value), so the launch sequence is fixed and no
+// kernel traps. Large fronts also record a row whose entries are larger than positive definiteness allows, before they
+// can leave the range of their digits.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -464,7 +466,7 @@ static void factor_body(gp_ctx* ctx, gp_factor_t* f) {
         ProfScope ps_(ctx, KC_TRSM, B * stp.trsm_flops);
         k_trsm64<<<dim3((unsigned)stp.trsm128_total, B), 256, TRSM_SMEM, st>>>(
             fronts, dp.step_pre + stp.pre_off + stp.nfront + 1, stp.nfront, stp.kb, dp, f->panels, PE, f->itile, IE,
-            f->rho, ps->n, f->op_maps, f->op_slot, f->tiles_err, f->wait_lim);
+            f->rho, ps->n, f->op_maps, f->op_slot, f->notpd, f->tiles_err, f->wait_lim);
         GP_CHECK_LAUNCH(ctx);
       }
       if (stp.group64.total > 0) update(stp.group64, stp.kb, true);

@@ -22,8 +22,11 @@
 // A step is a chain of dependent instructions (pivot, reciprocal root, scaling, one hand-over), so nothing else waits
 // for anything: every column of the factor and row of the inverse has a place and an mbarrier of its own, and the warp
 // that holds the next one updates and publishes it before it does the rest of its updates.
-// A pivot that is not positive, or an entry larger than its diagonals allow (either means that the tile is not
-// positive definite at or before that row), records its column and the elimination goes on with any value.
+// A pivot that is not positive, a diagonal that has fallen below zero before its turn or an entry larger than its diagonals
+// allow (each means that the tile is not positive definite at or before that row) records its row, and the elimination
+// goes on with any value. The smallest recorded column is the first failing one: what comes before it is positive
+// definite and within the ranges, and its own row either keeps to them, so that its pivot comes out right and not
+// positive, or is recorded where it leaves them.
 #pragma once
 #include "f64_digits.cuh"
 #include "gp_internal.cuh"
@@ -210,9 +213,11 @@ __device__ __forceinline__ void factor(Smem& sm, double* __restrict__ P, int64_t
     }
     __syncwarp();
     if (lane == 0) tcg::mbar_arrive_cluster(r_ready + k * 8);
-    const int64_t lim = 1LL << (60 - o.s);   // what the diagonals allow
-    if ((a0 >= lim || a0 <= -lim) && lane > k) atomicMin(flag, first + lane);
-    if ((a1 >= lim || a1 <= -lim) && lane + 32 > k) atomicMin(flag, first + lane + 32);
+    // what the diagonals allow: |a_ik| < sqrt(d) / 2 <= 2^-s, |l_ik| < 1/2
+    const int64_t lim = 1LL << (60 - o.s);
+    constexpr int half = (1 << 29) + 1;
+    if ((a0 >= lim || a0 <= -lim || abs(c0.x) > half) && lane > k) atomicMin(flag, first + lane);
+    if ((a1 >= lim || a1 <= -lim || abs(c1.x) > half) && lane + 32 > k) atomicMin(flag, first + lane + 32);
 #pragma unroll
     for (int q = 0; q < 3; q++) {
       H0[q] = H0[q + 1];
@@ -267,6 +272,14 @@ __device__ __forceinline__ void factor(Smem& sm, double* __restrict__ P, int64_t
       mad(H1[q], l1.x, -v[q].x);
       mad(C1[q], l1.x, -v[q].y);
       mad(C1[q], l1.y, -v[q].x);
+    }
+    if ((k & 15) == 15) {   // a diagonal below zero is seen before it can wrap: 16 columns take at most 4 of it
+#pragma unroll
+      for (int q = 0; q < 8; q++) {
+        const int j = jn + 8 * q;
+        const int64_t d = j < 32 ? H0[q & 3] + (C0[q & 3] >> 30) : H1[q] + (C1[q] >> 30);
+        if (j < bw && lane == (j & 31) && d < 0) atomicMin(flag, first + j);
+      }
     }
   }
   // L in FP64 (warp w the columns w + 8 q; every column has been waited for)

@@ -42,7 +42,8 @@ __device__ __forceinline__ void tmem_ld_levels(uint32_t ta, int ld, float (&a)[f
 // inverse's planes arrive by one bulk copy; 26 digit products of 128 x 64 x 64 follow, one TMEM accumulator per level;
 // each thread then rounds its row's entries of X to FP64 for the panel and cuts them into the digits the updates read (at
 // the row's scale rho), which leave through shared memory by TMA (a thread's own 16-byte stores would touch one line
-// each). Bounded by latency at the top levels (one wave of CTAs: load, cut, multiply, store in turn): 21 us a launch with
+// each). A row whose entries are more than its variance allows (|L_ij| <= sqrt(C_ii) <= 2^(rho + 1)) is not positive
+// definite at or before its own column and records it: its digits may have wrapped. Bounded by latency at the top levels (one wave of CTAs: load, cut, multiply, store in turn): 21 us a launch with
 // one tile, 117 us as an FP64 substitution column by column.
 constexpr int TRSM_ROWS = 128;
 constexpr int TRSM_PLANE_A = TRSM_ROWS * 128;   // bytes of one digit plane of B
@@ -52,7 +53,8 @@ __global__ void __launch_bounds__(256, 1)
     k_trsm64(const int32_t* __restrict__ fronts, const int64_t* __restrict__ pre, int nfront, int kb, DevPlan dp,
              double* __restrict__ panels, int64_t PE, const uint8_t* __restrict__ itile, int64_t IE,
              const int32_t* __restrict__ rho, int64_t n, const uint8_t* __restrict__ tmaps,
-             const int32_t* __restrict__ slot_of, int32_t* __restrict__ err, tcg::WaitLimit lim) {
+             const int32_t* __restrict__ slot_of, int32_t* __restrict__ notpd, int32_t* __restrict__ err,
+             tcg::WaitLimit lim) {
   using namespace f64d;
   extern __shared__ __align__(1024) uint8_t trsm_raw[];
   uint8_t* sm = (uint8_t*)(((uintptr_t)trsm_raw + 1023) & ~(uintptr_t)1023);
@@ -84,7 +86,8 @@ __global__ void __launch_bounds__(256, 1)
   const bool rok = row < nr;
   double* P = panels + (int64_t)b * PE + dp.loff[s] + (int64_t)(c0 + 32 * half) * m + r0 + row;   // this thread's entries
   const int nc = min(max(bw - 32 * half, 0), rok ? 32 : 0);
-  const int32_t rr = rok ? rho[(int64_t)b * n + dp.frows[dp.frow_off[s] + r0 + row]] : 0;
+  const int32_t col = rok ? dp.frows[dp.frow_off[s] + r0 + row] : 0;   // the row's own (permuted) column
+  const int32_t rr = rok ? rho[(int64_t)b * n + col] : 0;
   int rx;
   {
     double x[32];
@@ -141,6 +144,7 @@ __global__ void __launch_bounds__(256, 1)
   ok = ok && !skip;
   __syncwarp();
   tcg::tc_fence_after();
+  bool over = rx > rr + 1;   // |B_c| 2^-sigma_c < 2^rr in a positive definite matrix
   {
     double* p = P;
 #pragma unroll 1
@@ -151,13 +155,14 @@ __global__ void __launch_bounds__(256, 1)
 #pragma unroll
       for (int c = 0; c < 8; c++, p += m) {
         const float al[NL] = {a[0][c], a[1][c], a[2][c], a[3][c], a[4][c], a[5][c], a[6][c]};
-        const Norm x = product_any(al, rx + einv[32 * half + 8 * g + c], rr + 1);
+        const Norm x = product_any(al, rx + einv[32 * half + 8 * g + c], rr + 1, over);
         if (ok && 8 * g + c < nc) *p = to_double(x);
         v[c] = to_biased(x, rr);
       }
       store8(sm + row * 128 + (((4 * half + g) ^ (row & 7)) << 4), TRSM_PLANE_A, v);
     }
   }
+  if (ok && rok && over) atomicMin(notpd + b, col);
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");
   tcg::tc_fence_before();
   __syncthreads();

@@ -1,0 +1,124 @@
+"""The FP64 path at the edges of its fixed-point arithmetic, through the C-ABI."""
+import math
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2411_05869_gb300 import synth
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA device")]
+
+
+def _dev(a):
+    return torch.as_tensor(np.ascontiguousarray(a), dtype=torch.float64, device="cuda")
+
+
+def _first_failing(C):
+    """The first column whose pivot is not positive (None: positive definite), with pivots well away from zero."""
+    A = C.copy()
+    for k in range(len(A)):
+        assert abs(A[k, k]) > 1e-9 * C[k, k]
+        if A[k, k] <= 0:
+            return k
+        c = A[k + 1:, k] / math.sqrt(A[k, k])
+        A[k + 1:, k + 1:] -= np.outer(c, c)
+    return None
+
+
+def _hyper(amplitude, core_var, r0, noise, r=0.1):
+    return synth.Hyper(d=2, n1=1, n2=1, bump_dims=2, core_var=core_var, core_radius=np.full(2, 50.0), s0=0.0 if core_var < 0 else 1.0,
+                       r0=np.full(2, r0), h=np.array([0.5, 0.5]), a=np.array([amplitude]), b=np.ones(1), r=np.full(1, r),
+                       noise_var=noise)
+
+
+def _grid(n, seed, jitter=0.2):
+    rng = np.random.default_rng(seed)
+    k = math.ceil(math.sqrt(n))
+    g = np.stack(np.meshgrid(np.arange(k), np.arange(k)), -1).reshape(-1, 2)[:n]
+    return (g + 0.5 + rng.uniform(-jitter, jitter, g.shape)) / k
+
+
+def _check_flags(X, settings):
+    """Batch of a good setting and `settings`: the flagged columns are the dense Cholesky's first failing pivots."""
+    from paper_2411_05869_gb300 import gp
+    n = len(X)
+    good = _hyper(0.5, 1.0, 0.03, 0.3)
+    hs = [good] + settings
+    ctx = gp.Context(0)
+    ps = ctx.assemble(_dev(X), good.core_radius)
+    perm = ps.export("perm")
+    want = [_first_failing(oracle.dense_cov(h, X)[np.ix_(perm, perm)]) for h in hs]
+    f = ctx.factor(ps, hs, gp.GP_FP64)
+    ll = f.loglik(_dev(np.ones((len(hs), n)))).cpu().numpy()
+    info = f.info()
+    got = [None if c < 0 else int(c) for c in info["not_pd_column"]]
+    f.free()
+    ps.free()
+    assert got == want
+    for v, w in zip(ll, want):
+        assert v == -np.inf if w is not None else np.isfinite(v)
+    return want
+
+
+@pytest.mark.parametrize("noise", [-0.05, -0.9])
+@pytest.mark.parametrize("n", [200, 600])
+def test_pair_that_breaks_definiteness_is_flagged_at_its_own_column(n, noise):
+    """Nearly uncorrelated points but one close pair, and a negative noise: the pair's later column fails, by a little or by
+    far (its rows of L are then many times what their variances allow)."""
+    seen = set()
+    for seed in range(6):
+        X = _grid(n, seed)
+        rng = np.random.default_rng(100 + seed)
+        i, j = rng.choice(n, 2, replace=False)
+        X[i] = X[j] + 1e-4
+        want = _check_flags(X, [_hyper(0.0, 1.0, 0.02, noise)])
+        assert want[0] is None and want[1] is not None
+        seen.add(want[1] // 64)
+    assert len(seen) > 1   # several block columns
+
+
+@pytest.mark.parametrize("ring", [40, 70, 120, 180, 240])
+def test_variance_far_below_its_columns_share_is_flagged(ring):
+    """C = tau^2 I - c f f^T with f large at one point: its row of L is as long as its variance allows in every column, and
+    their squares add up to many times that."""
+    n, radius = 320, 0.1
+    rng = np.random.default_rng(ring)
+    X = rng.uniform(3.0, 3.3, (n, 2))   # outside the bump
+    phi = np.linspace(0, 2 * math.pi, ring, endpoint=False) + 0.01
+    where = rng.permutation(n)
+    X[where[:ring]] = 0.5 + radius * np.stack([np.cos(phi), np.sin(phi)], -1)
+    X[where[ring]] = 0.5
+    settings = []
+    for share in (0.3, 0.45, 0.6, 0.75, 0.9):    # c |f_ring|^2: the ring alone is positive definite
+        for var in (0.5, 0.1, 0.02, 0.004):      # 1 - c f_middle^2, the middle's variance (tau^2 = 1)
+            c = 1 - var
+            fk = math.sqrt(share / (c * ring))   # f on the ring: exp(1 - 1 / (1 - t))
+            t = 1 - 1 / (1 - math.log(fk))
+            settings.append(_hyper(1.0, -c, 0.02, 1.0, r=radius / math.sqrt(t)))
+    want = _check_flags(X, settings)
+    assert sum(w is not None for w in want) >= 10
+
+
+def test_sparse_fronts_report_the_first_failing_column():
+    from paper_2411_05869_gb300 import gp
+    w = synth.spatial_2d(n=2500, m=1, seed=5, rho=0.15, noise_var=0.05)
+    bad = w.hyper.copy()
+    bad.noise_var = -2e-4
+    ctx = gp.Context(0)
+    ps = ctx.assemble(_dev(w.X), w.hyper.core_radius)
+    perm = ps.export("perm")
+    C = oracle.dense_cov(bad, w.X)[np.ix_(perm, perm)]
+    A = C.copy()
+    want = None
+    for k in range(len(A)):
+        if A[k, k] <= 0:
+            want = k
+            break
+        c = A[k + 1:, k] / math.sqrt(A[k, k])
+        nz = np.flatnonzero(c)
+        A[np.ix_(k + 1 + nz, k + 1 + nz)] -= np.outer(c[nz], c[nz])
+    f = ctx.factor(ps, [w.hyper, bad], gp.GP_FP64)
+    cols = f.info()["not_pd_column"]
+    assert cols[0] == -1 and want is not None and cols[1] == want

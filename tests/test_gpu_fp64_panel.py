@@ -60,3 +60,80 @@ def test_inverse_whose_low_halves_have_one_sign(panel, low, terms):
     assert bad is None
     E = np.abs(D.astype(np.longdouble) @ P.astype(np.longdouble) - np.eye(64))
     assert (E <= 2.0 ** -49 * np.abs(D).max(1, keepdims=True)).all(), float(E.max())
+
+
+def _first_failing(A):
+    """First column whose pivot is not positive (None: positive definite); pivots are away from zero by construction."""
+    A = A.astype(np.longdouble)
+    for k in range(len(A)):
+        if not A[k, k] > 0:
+            return k
+        c = A[k + 1:, k] / np.sqrt(A[k, k])
+        A[k + 1:, k + 1:] -= np.outer(c, c)
+    return None
+
+
+@pytest.mark.parametrize("p", [1, 15, 16, 31, 32, 47, 63])
+@pytest.mark.parametrize("scale", [1.0, 3.9])   # the ends of the rows' fixed-point range
+def test_row_of_a_tile_that_breaks_definiteness_is_its_first_failing_column(panel, p, scale):
+    """Uncorrelated columns and one row with the same entry in each: its pivot falls by r^2 per column, to below zero by a
+    little, to any number of turns of a 64-bit integer, or to values beyond the fixed point."""
+    for r in np.concatenate([np.linspace(0.05, 2.0, 80), [5.0, 30.0, 1e3, 1e6, 1e9, 1e30, 1e100]]):
+        if abs(p * r * r - 1) < 1e-6:
+            continue
+        A = np.eye(64)
+        A[p, :p] = r
+        A *= scale
+        want = p if p * r * r > 1 else None
+        P, D, bad = panel(A, np.diag(A))
+        assert bad == want, (p, r, bad)
+        if bad is None:
+            assert np.abs(P @ P.T - (A + np.tril(A, -1).T)).max() <= 64 * 2.0 ** -50 * scale
+
+
+@pytest.mark.parametrize("bw", [1, 17, 33, 64])
+def test_random_tiles_report_the_first_failing_pivot(panel, bw):
+    rng = np.random.default_rng(bw)
+    for k in range(40):
+        Q = np.linalg.qr(rng.standard_normal((bw, bw)))[0]
+        ev = np.exp(rng.uniform(-6, 0, bw))
+        ev[rng.integers(bw)] *= rng.choice([-1.0, 1.0])
+        d = 2.0 ** rng.integers(-20, 20, bw)
+        A = (Q * ev) @ Q.T
+        A = (A + A.T) / 2
+        want = _first_failing(A)
+        A = A * d[:, None] * d[None, :]
+        P, D, bad = panel(np.tril(A), np.abs(np.diag(A)) + (np.diag(A) == 0))
+        assert bad == want
+
+
+@pytest.mark.parametrize("rows", [1, 64, 65, 128, 300])
+def test_rows_below_are_flagged_only_beyond_their_variance(panel, rows):
+    """A row of L longer than sqrt(C_ii) shows at its own pivot; one with an entry of many times that is recorded here."""
+    rng = np.random.default_rng(rows)
+    base = np.concatenate([np.eye(64), np.zeros((rows, 64))])
+    diag = np.concatenate([np.ones(64), 10.0 ** rng.uniform(-3, 3, rows)])
+    base[64:] = rng.uniform(-0.99, 0.99, (rows, 64)) * np.sqrt(diag[64:, None])
+    P, D, bad = panel(base, diag)
+    assert bad is None
+    assert np.array_equal(P[64:], base[64:]) or np.abs(P[64:] - base[64:]).max() <= 2.0 ** -53 * np.sqrt(diag.max())
+    for factor in (8.0, 1e3, 1e9, 1e40, 1e200):
+        for col in (0, 31, 32, 63):
+            i, j = rng.integers(rows), rng.integers(rows)
+            A = base.copy()
+            A[64 + i, col] = factor * math.sqrt(diag[64 + i])
+            A[64 + j, col] = -factor * math.sqrt(diag[64 + j])
+            P, D, bad = panel(A, diag)
+            assert bad == 64 + min(i, j), (factor, col)
+
+
+@pytest.mark.parametrize("kappa", [1e2, 1e6, 1e10, 1e13])
+def test_ill_conditioned_positive_definite_panels_are_not_flagged(panel, kappa):
+    rng = np.random.default_rng(int(math.log10(kappa)))
+    for k in range(10):
+        n = 64 + 150
+        x = np.sort(rng.uniform(0, 1, n))
+        K = np.exp(-0.5 * ((x[:, None] - x[None]) / 0.3) ** 2) + (10.0 / kappa) * np.eye(n)
+        K *= 10.0 ** rng.uniform(-8, 8)
+        P, D, bad = panel(np.concatenate([np.tril(K[:64, :64]), K[64:, :64]]), np.diag(K))
+        assert bad is None
