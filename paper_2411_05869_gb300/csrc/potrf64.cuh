@@ -25,7 +25,7 @@
 // A pivot that is not positive, a diagonal that has fallen below zero before its turn or an entry larger than its diagonals
 // allow (each means that the tile is not positive definite at or before that row) records its row, and the elimination
 // goes on with any value. The smallest recorded column is the first failing one: what comes before it is positive
-// definite and within the ranges, and its own row either keeps to them, so that its pivot comes out right and not
+// definite and within the ranges (an infinite variance is taken as 2^1024, and its root written as infinite), and its own row either keeps to them, so that its pivot comes out right and not
 // positive, or is recorded where it leaves them.
 #pragma once
 #include "f64_digits.cuh"
@@ -49,6 +49,10 @@ struct Smem {               // of either CTA; the factor's CTA writes its column
   int sigma[PT];
   uint64_t lready[PT], rready[PT], xready[PT];   // mbarriers: lc[k]; R[k] and rs[k]; xr[k] and xe[k] are in
 };
+
+// A row's sigma for an infinite variance (an exponent field of 0x7ff).
+constexpr int SIGMA_INF = ((0x7ff - 1021) >> 1) + 1;
+__device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0x7ff00000) != 0x7ff00000; }
 
 // x 2^(60 - e) to within a unit, |x| <= 2^(e - 2) in a positive definite tile; at least 2^60 in magnitude for |x| >= 2^e.
 __device__ __forceinline__ int64_t double2fix60(double x, int e) {
@@ -179,11 +183,11 @@ __device__ __forceinline__ void factor(Smem& sm, double* __restrict__ P, int64_t
       const int sj = sm.sigma[w + 8 * q];
       if (q < 4) {
         H0[q] = double2fix60(x0[q], s0 + sj);
-        bad0 = bad0 || H0[q] >= 1LL << 60 || H0[q] < -(1LL << 60);
+        bad0 = bad0 || H0[q] >= 1LL << 60 || H0[q] < -(1LL << 60) || (!finite(x0[q]) && w + 8 * q != lane);
         C0[q] = 0;
       }
       H1[q] = double2fix60(x1[q], s1 + sj);
-      bad1 = bad1 || H1[q] >= 1LL << 60 || H1[q] < -(1LL << 60);
+      bad1 = bad1 || H1[q] >= 1LL << 60 || H1[q] < -(1LL << 60) || (!finite(x1[q]) && w + 8 * q != lane + 32);
       C1[q] = 0;
     }
     if (bad0) atomicMin(flag, first + lane);
@@ -288,7 +292,10 @@ __device__ __forceinline__ void factor(Smem& sm, double* __restrict__ P, int64_t
 #pragma unroll
     for (int p = 0; p < 2; p++) {
       const int i = lane + 32 * p;
-      if (j <= i && i < bw) P[j * ld + i] = f64d::fix2double(join30(sm.lc[j][i]), sm.sigma[i] - 60);
+      if (j <= i && i < bw) {
+        const double l = f64d::fix2double(join30(sm.lc[j][i]), sm.sigma[i] - 60);
+        P[j * ld + i] = i == j && sm.sigma[i] == SIGMA_INF ? __longlong_as_double(0x7ff0000000000000LL) : l;
+      }
     }
 }
 

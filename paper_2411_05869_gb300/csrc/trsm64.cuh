@@ -89,6 +89,7 @@ __global__ void __launch_bounds__(256, 1)
   const int32_t col = rok ? dp.frows[dp.frow_off[s] + r0 + row] : 0;   // the row's own (permuted) column
   const int32_t rr = rok ? rho[(int64_t)b * n + col] : 0;
   int rx;
+  bool over = false;   // more than the row's variance allows
   {
     double x[32];
     const double* p = P;
@@ -104,6 +105,7 @@ __global__ void __launch_bounds__(256, 1)
     for (int c = 0; c < 32; c++) {
       const int e = (__double2hiint(x[c]) >> 20) & 0x7ff;
       ex = max(ex, e == 0 ? -4096 : e - einv[p64::PT + 32 * half + c]);
+      over = over || e == 0x7ff;
     }
     emax_s[half][row] = ex;
     __syncthreads();
@@ -144,7 +146,7 @@ __global__ void __launch_bounds__(256, 1)
   ok = ok && !skip;
   __syncwarp();
   tcg::tc_fence_after();
-  bool over = rx > rr + 1;   // |B_c| 2^-sigma_c < 2^rr in a positive definite matrix
+  over = over || rx > rr + 1;   // |B_c| 2^-sigma_c < 2^rr in a positive definite matrix
   {
     double* p = P;
 #pragma unroll 1

@@ -122,3 +122,32 @@ def test_sparse_fronts_report_the_first_failing_column():
     f = ctx.factor(ps, [w.hyper, bad], gp.GP_FP64)
     cols = f.info()["not_pd_column"]
     assert cols[0] == -1 and want is not None and cols[1] == want
+
+
+@pytest.mark.parametrize("where", ["alone", "pair", "pair_apart"])
+def test_infinite_covariances(where):
+    """A bump whose square overflows. One point inside: its variance is infinite, so is the log-determinant, and nothing
+    else is affected; no pivot fails. Two points inside: their covariance is infinite too, and the later one fails."""
+    from paper_2411_05869_gb300 import gp
+    n = 300
+    X = _grid(n, 3)
+    d = np.linalg.norm(X - 0.5, axis=1)
+    i, j = np.argsort(d)[:2]
+    X[i] = 0.5
+    if where != "alone":
+        X[j] = 0.503
+    huge = _hyper(1e160, 1.0, 0.03, 0.3, r=0.006)
+    if where == "pair_apart":   # one point changes places with the pair's: other columns of the elimination order
+        huge.h = huge.h * 0 + X[0]
+        X[1] = X[0] + 0.003
+    inside = np.flatnonzero(np.linalg.norm(X - huge.h, axis=1) < 0.006)
+    assert len(inside) == (1 if where == "alone" else 2)
+    good = _hyper(0.5, 1.0, 0.03, 0.3, r=0.006)
+    good.h = huge.h.copy()
+    ctx = gp.Context(0)
+    ps = ctx.assemble(_dev(X), good.core_radius)
+    f = ctx.factor(ps, [good, huge], gp.GP_FP64)
+    ll = f.loglik(_dev(np.ones((2, n)))).cpu().numpy()
+    pos = np.argsort(ps.export("perm"))[inside]
+    assert np.isfinite(ll[0]) and ll[1] == -np.inf
+    assert list(f.info()["not_pd_column"]) == [-1, -1 if where == "alone" else pos.max()]
