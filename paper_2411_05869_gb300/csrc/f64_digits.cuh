@@ -33,15 +33,22 @@ __device__ __forceinline__ int rho_of(double x) {
 // the digits are the entry rounded); digit 0 is what is left above bit 52.
 constexpr int64_t BIAS = 64 + ((256LL << 7) | (256LL << 16) | (256LL << 25) | (256LL << 34) | (256LL << 43));
 
+// The significand of x at bit 62 and the exponent field that goes with it, zeros and numbers below the normal range as they
+// are: |x| = man 2^(e - 1085).
+__device__ __forceinline__ uint64_t significand(double x, int& e) {
+  const int hi = __double2hiint(x), f = (hi >> 20) & 0x7ff;
+  const uint32_t mh = (uint32_t)(hi & 0xfffff) | (uint32_t)min(f, 1) << 20, ml = (uint32_t)__double2loint(x);
+  e = max(f, 1);
+  return ((uint64_t)__funnelshift_l(ml, mh, 10) << 32) | (ml << 10);
+}
+
 // x at scale 2^rho, |x| <= 2^(rho + 1), plus BIAS (larger |x|, which only a failed factorization has, come out wrong).
 // The sign is applied as a complement: one unit of 2^-61 off for negative x.
 __device__ __forceinline__ int64_t to_biased(double x, int rho) {
-  const int hi = __double2hiint(x);
-  const uint32_t mh = (uint32_t)(hi & 0xfffff) | 0x100000u, ml = (uint32_t)__double2loint(x);
-  const int n = min(max(1024 + rho - ((hi >> 20) & 0x7ff), 0), 63);   // right shift of the significand at bit 62
-  const uint64_t man = ((uint64_t)__funnelshift_l(ml, mh, 10) << 32) | (ml << 10);
-  const int64_t sg = (int64_t)(hi >> 31);
-  return ((int64_t)(man >> n) ^ sg) + BIAS;
+  int e;
+  const uint64_t man = significand(x, e);
+  const int n = min(max(1024 + rho - e, 0), 63);   // right shift
+  return ((int64_t)(man >> n) ^ (int64_t)(__double2hiint(x) >> 31)) + BIAS;
 }
 
 // Digits s of two biased entries as a pair of FP16 numbers: 0x6400 + u is the FP16 number 1024 + u, u = d + 256.
@@ -94,12 +101,17 @@ __device__ __forceinline__ Norm normalise(int64_t v, int e0) {
   r.e = e0 - z;
   return r;
 }
-// Rounded to FP64 (half away from zero; below the normal range: 0), in integers: the FP64 pipe is the slow one here.
+// Rounded to FP64 (half away from zero), in integers: the FP64 pipe is the slow one here.
 __device__ __forceinline__ double to_double(const Norm& r) {
-  const uint64_t man = (r.n + 512) >> 10;   // 2^52 <= man <= 2^53
-  const int E = 1022 + r.e;                 // the biased exponent less one: man brings the other one
+  uint64_t man = (r.n + 512) >> 10;   // 2^52 <= man <= 2^53
+  int E = 1022 + r.e;                 // the biased exponent less one: man brings the other one
+  if (E < 0) {                        // below the normal range: man in units of 2^-1074, without a leading one of its own
+    const int n = 10 - max(E, -53);
+    man = (r.n + (1ull << (n - 1))) >> n;
+    E = 0;
+  }
   uint32_t hi = (uint32_t)(man >> 32) + ((uint32_t)min(E, 2045) << 20), lo = (uint32_t)man;
-  const bool zero = r.n == 0 || E <= 0;
+  const bool zero = r.n == 0;
   hi = zero ? 0u : hi | ((uint32_t)r.sg & 0x80000000u);
   lo = zero ? 0u : lo;
   return __hiloint2double((int)hi, (int)lo);

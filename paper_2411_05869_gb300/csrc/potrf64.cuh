@@ -56,11 +56,10 @@ __device__ __forceinline__ bool finite(double x) { return (__double2hiint(x) & 0
 
 // x 2^(60 - e) to within a unit, |x| <= 2^(e - 2) in a positive definite tile; at least 2^60 in magnitude for |x| >= 2^e.
 __device__ __forceinline__ int64_t double2fix60(double x, int e) {
-  const int hi = __double2hiint(x);
-  const uint32_t mh = (uint32_t)(hi & 0xfffff) | 0x100000u, ml = (uint32_t)__double2loint(x);
-  const int n = min(max(1025 + e - ((hi >> 20) & 0x7ff), 0), 63);   // right shift of the significand at bit 62
-  const uint64_t man = ((uint64_t)__funnelshift_l(ml, mh, 10) << 32) | (ml << 10);
-  return (int64_t)(man >> n) ^ (int64_t)(hi >> 31);
+  int f;
+  const uint64_t man = f64d::significand(x, f);
+  const int n = min(max(1025 + e - f, 0), 63);   // right shift
+  return (int64_t)(man >> n) ^ (int64_t)(__double2hiint(x) >> 31);
 }
 
 // The reciprocal root of a pivot 0 < d < 2^60 (units of 2^-60): d 2^-60 = m 4^(1 - s), 1/4 <= m < 1, 1 / sqrt(d) = r

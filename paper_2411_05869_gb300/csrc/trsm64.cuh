@@ -104,12 +104,12 @@ __global__ void __launch_bounds__(256, 1)
 #pragma unroll
     for (int c = 0; c < 32; c++) {
       const int e = (__double2hiint(x[c]) >> 20) & 0x7ff;
-      ex = max(ex, e == 0 ? -4096 : e - einv[p64::PT + 32 * half + c]);
+      ex = max(ex, max(e, 1) - einv[p64::PT + 32 * half + c]);
       over = over || e == 0x7ff;
     }
     emax_s[half][row] = ex;
     __syncthreads();
-    rx = max(max(ex, emax_s[half ^ 1][row]) - 1022, -900);   // |x| 2^-sigma < 2^rx
+    rx = max(ex, emax_s[half ^ 1][row]) - 1022;   // |x| 2^-sigma < 2^rx
 #pragma unroll
     for (int g = 0; g < 4; g++) {
       int64_t v[8];

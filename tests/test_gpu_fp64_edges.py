@@ -151,3 +151,22 @@ def test_infinite_covariances(where):
     pos = np.argsort(ps.export("perm"))[inside]
     assert np.isfinite(ll[0]) and ll[1] == -np.inf
     assert list(f.info()["not_pd_column"]) == [-1, -1 if where == "alone" else pos.max()]
+
+
+@pytest.mark.parametrize("k", [-960, -1000, -40, 900])
+@pytest.mark.parametrize("n", [200, 513])
+def test_covariances_of_any_scale(n, k):
+    """C times 2^k and r times 2^(k / 2) move the log-likelihood by -n k / 2 log 2 and nothing else: the entries of C keep
+    their digits, down to 2^-74 of the variances where 2^-1000 leaves the normal range."""
+    from paper_2411_05869_gb300 import gp
+    w = synth.spatial_2d(n=n, m=1, seed=70 + n, rho=2.0, noise_var=0.1)
+    h = w.hyper.copy()
+    h.core_var, h.noise_var = math.ldexp(h.core_var, k), math.ldexp(h.noise_var, k)
+    ctx = gp.Context(0)
+    ps = ctx.assemble(_dev(w.X), w.hyper.core_radius)
+    f = ctx.factor(ps, [w.hyper, h], gp.GP_FP64)
+    ll = f.loglik(_dev(np.stack([w.normals, w.normals * 2.0 ** (k // 2)]))).cpu().numpy()
+    want = ll[0] - 0.5 * n * k * math.log(2.0)
+    # kappa <= 1e5 here: the quadratic form and the log-determinant are good to n kappa 2^-53 < 1e-8 at worst; a backward
+    # error of 2^-53 in general position gives about sqrt(n) kappa 2^-53 of the quadratic form
+    assert abs(ll[1] - want) <= 1e-11 * max(abs(want), abs(ll[0])), (ll, want)
