@@ -140,16 +140,39 @@ __device__ __forceinline__ Norm product_rows(const float (&a)[NL], int e) {
   const float a0 = fminf(fmaxf(a[0], -0x1p21f), 0x1p21f);
   return normalise(high_levels(a0, a[1], a[2], a[3]) * (1LL << 14) + (int64_t)__float2int_rn(low), e + 3);
 }
-// A dot product of 64 terms of at most 1 that the caller knows to be at most 2^eb: units of 2^(eb - 61) where the levels
-// give that much, 2^-55 of the scales at the coarsest (the 64 terms' bound), 2^-69 at the finest. Sets `over` where it is
-// more than 1.5 times 2^eb (levels 0 and 1 tell, to 2^-12); the result is then any number.
-__device__ __forceinline__ Norm product_any(const float (&a)[NL], int e, int eb, bool& over) {
-  const int S = 16 - max(min(eb - e, 6), -8);   // extra bits below the levels 0..3
-  const float low = fmaf(a[6], 0x1p-27f, a[5] * 0x1p-18f) * __int_as_float((127 + S) << 23);
+// A dot product of 64 terms of at most 2^e each, cut to units of 2^(rho - 61), from all levels or from the levels 0..3. Sets
+// `over` where it is more than 1.5 times 2^(rho + 1) (levels 0 and 1 tell, to 2^-12); the result is then any number.
+__device__ __forceinline__ int64_t product_fixed(const float (&a)[NL], int e, int rho, bool all, bool& over) {
+  const int S = 15 - max(min(rho - e, 5), -9);   // bits kept below levels 0..3: at most 62 in all
   over = over || fabsf(fmaf(a[1], 0x1p-9f, a[0])) > 1.5f * __int_as_float((127 + 34 - S) << 23);
   int64_t v = high_levels(a[0], a[1], a[2], a[3]) << S;
-  v += (int64_t)__float2int_rn(a[4]) * (int64_t)(1 << (S - 9));
-  return normalise(v + (int64_t)__float2int_rn(low), e + 17 - S);
+  if (all) {
+    const float low = fmaf(a[6], 0x1p-27f, a[5] * 0x1p-18f) * __int_as_float((127 + S) << 23);
+    v += (int64_t)__float2int_rn(a[4]) * (int64_t)(1 << (S - 9)) + (int64_t)__float2int_rn(low);
+  }
+  const int n = rho - 61 - (e - 45 - S);   // from units of 2^(e - 45 - S)
+  return n >= 0 ? v >> min(n, 63) : v << min(-n, 63);
+}
+
+// For a residual in 64-bit integers modulo 2^64, which is right wherever the residual itself is small: a dot product in
+// units of 2^-72 of its scales, and x in units of 2^u.
+__device__ __forceinline__ uint64_t product_mod72(const float (&a)[NL]) {
+  int64_t low = (int64_t)__float2int_rn(a[4]) * (1 << 18);
+  low += (int64_t)__float2int_rn(a[5]) * (1 << 9);
+  low += (int64_t)__float2int_rn(a[6]);
+  return ((uint64_t)high_levels(a[0], a[1], a[2], a[3]) << 27) + (uint64_t)low;
+}
+__device__ __forceinline__ uint64_t fixed_mod(double x, int u) {
+  int e;
+  const uint64_t man = significand(x, e) >> 10;   // |x| = man 2^(e - 1075)
+  const int n = e - 1075 - u;
+  const uint64_t v = n >= 0 ? (n < 64 ? man << n : 0) : man >> min(-n, 63);
+  return __double2hiint(x) < 0 ? 0 - v : v;
+}
+// What the first six or four digits of a biased entry say: the entry in units of 2^-61 of its scale, cut to 2^-54 or 2^-36.
+__device__ __forceinline__ int64_t digits_of(int64_t v, bool six) {
+  constexpr int64_t OFF = BIAS - 64;   // 256 in every field
+  return six ? (v & ~((1LL << 7) - 1)) - OFF : (v & ~((1LL << 25) - 1)) - (OFF & ~((1LL << 25) - 1));
 }
 
 }  // namespace f64d

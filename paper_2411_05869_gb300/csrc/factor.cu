@@ -464,7 +464,7 @@ static void factor_body(gp_ctx* ctx, gp_factor_t* f) {
       }
       if (stp.trsm128_total > 0) {
         ProfScope ps_(ctx, KC_TRSM, B * stp.trsm_flops);
-        k_trsm64<<<dim3((unsigned)stp.trsm128_total, B), 256, TRSM_SMEM, st>>>(
+        k_trsm64<<<dim3((unsigned)stp.trsm128_total, B), TRSM_THREADS, TRSM_SMEM, st>>>(
             fronts, dp.step_pre + stp.pre_off + stp.nfront + 1, stp.nfront, stp.kb, dp, f->panels, PE, f->itile, IE,
             f->rho, ps->n, f->op_maps, f->op_slot, f->notpd, f->tiles_err, f->wait_lim);
         GP_CHECK_LAUNCH(ctx);

@@ -38,7 +38,8 @@ namespace p64 {
 constexpr int PT = GP_TILE;
 constexpr int THREADS = 256;   // per CTA
 constexpr int PLANE = PT * 128;                       // bytes of one digit plane of the inverse (64 rows of 64 FP16)
-constexpr int TILE_BYTES = f64d::NS * PLANE + 2 * PT * 4;   // the planes, the rows' exponents and the columns' sigma
+constexpr int TILE_BYTES = 2 * f64d::NS * PLANE + 2 * PT * 4;   // the inverse's planes, the factor's, the inverse's rows'
+                                                                // exponents and its columns' (the factor's rows') sigma
 
 struct Smem {               // of either CTA; the factor's CTA writes its columns into both
   int2 lc[PT][PT];          // column k of the factor: (lh, ll) of every row
@@ -144,11 +145,12 @@ __device__ __forceinline__ void wait_cluster(uint64_t* bar, int32_t* err) {
   __syncwarp();
 }
 
-// The elimination (the cluster's first CTA): P points at the tile's entry (0, 0), column stride ld; L replaces it. Warp w holds
+// The elimination (the cluster's first CTA): P points at the tile's entry (0, 0), column stride ld; L replaces it, and its
+// digit planes go to `planes`, row i at scale 2^(sigma_i - 2) (128-byte-swizzled tiles of 64 rows x 64 FP16). Warp w holds
 // the columns w + 8 q, lane l the rows l (H0, C0; columns below 32 only) and l + 32 (H1, C1) of them; a finished column
 // is shifted out, so that entry 0 is always the warp's next column.
-__device__ __forceinline__ void factor(Smem& sm, double* __restrict__ P, int64_t ld, int bw, int32_t first,
-                                       int32_t* __restrict__ flag, int32_t* __restrict__ err) {
+__device__ __forceinline__ void factor(Smem& sm, double* __restrict__ P, int64_t ld, uint8_t* __restrict__ planes, int bw,
+                                       int32_t first, int32_t* __restrict__ flag, int32_t* __restrict__ err) {
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int64_t H0[4], C0[4], H1[8], C1[8];
   {
@@ -296,6 +298,17 @@ __device__ __forceinline__ void factor(Smem& sm, double* __restrict__ P, int64_t
         P[j * ld + i] = i == j && sm.sigma[i] == SIGMA_INF ? __longlong_as_double(0x7ff0000000000000LL) : l;
       }
     }
+#pragma unroll 1
+  for (int e = threadIdx.x; e < PT * PT / 8; e += THREADS) {   // eight columns of a row
+    const int i = e & (PT - 1), g = e / PT;
+    int64_t v[8];
+#pragma unroll
+    for (int c = 0; c < 8; c++) {
+      const int j = 8 * g + c;
+      v[c] = (j <= i && i < bw ? 8 * join30(sm.lc[j][i]) : 0) + f64d::BIAS;
+    }
+    f64d::store8(planes + i * 128 + ((g ^ (i & 7)) << 4), PLANE, v);
+  }
 }
 
 // The inverse (the cluster's second CTA): warp w holds the rows w + 8 r, lane l the columns l and l + 32; a finished row is
@@ -316,7 +329,7 @@ __device__ __forceinline__ void inverse(Smem& sm, double* __restrict__ DI, uint8
     }
   wait_cluster(&sm.rready[0], err);   // the scales are in, too
   const int sj[2] = {sm.sigma[lane], sm.sigma[lane + 32]};
-  int32_t* ex = reinterpret_cast<int32_t*>(tile + f64d::NS * PLANE);
+  int32_t* ex = reinterpret_cast<int32_t*>(tile + 2 * f64d::NS * PLANE);
   int64_t x[2] = {0, 0};
   int xe = 0;
   // Row k (entry 0 of its warp, all earlier rows applied), scaled and out to the other warps; R, rs: its pivot's root.
@@ -499,9 +512,11 @@ __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(p64::THREADS, 1)
   if (threadIdx.x < 3 * p64::PT) tcg::mbar_init(&sm.lready[threadIdx.x], 1);   // the three arrays
   asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
   tcg::cluster_sync();
-  if (tcg::cluster_ctarank() == 0) p64::factor(sm, P, m, bw, first, notpd + b, err);
-  else p64::inverse(sm, dinv + (int64_t)b * DE + dp.doff[s] + (int64_t)kb * p64::PT * p64::PT,
-                    itile + (int64_t)b * IE + (int64_t)fi * p64::TILE_BYTES, bw, err);
+  uint8_t* tile = itile + (int64_t)b * IE + (int64_t)fi * p64::TILE_BYTES;
+  if (tcg::cluster_ctarank() == 0)
+    p64::factor(sm, P, m, tile + f64d::NS * p64::PLANE, bw, first, notpd + b, err);
+  else
+    p64::inverse(sm, dinv + (int64_t)b * DE + dp.doff[s] + (int64_t)kb * p64::PT * p64::PT, tile, bw, err);
   tcg::cluster_sync();   // no CTA leaves while the other may write into it
 }
 

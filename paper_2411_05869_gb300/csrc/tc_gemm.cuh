@@ -204,14 +204,14 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
                : "memory");
 }
 // 4-D tiled TMA store from shared memory (elements outside the tensor are not written), and the wait of the issuing
-// thread until all its stores are done.
+// thread until all its stores have read their shared memory (they land before the kernel has ended).
 __device__ __forceinline__ void tma_store_4d(const void* tmap, int x, int y, int z, int w, uint32_t src) {
   asm volatile("cp.async.bulk.tensor.4d.global.shared::cta.bulk_group [%0, {%1, %2, %3, %4}], [%5];\n" ::"l"(tmap),
                "r"(x), "r"(y), "r"(z), "r"(w), "r"(src)
                : "memory");
 }
 __device__ __forceinline__ void bulk_store_wait() {
-  asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group 0;\n" ::: "memory");
+  asm volatile("cp.async.bulk.commit_group;\ncp.async.bulk.wait_group.read 0;\n" ::: "memory");
 }
 
 __device__ __forceinline__ uint32_t cluster_ctarank() {

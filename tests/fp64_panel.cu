@@ -72,7 +72,7 @@ extern "C" __attribute__((visibility("default"))) int fp64_panel(double* panel, 
   const int64_t PE = (int64_t)m * bw;
   k_potrf64<<<dim3(2, 1), p64::THREADS, sizeof(p64::Smem)>>>(fronts, 0, dp, P, PE, notpd, D, 4096, tile, p64::TILE_BYTES, err);
   if (nt > 0)
-    k_trsm64<<<dim3(nt, 1), 256, TRSM_SMEM>>>(fronts, d_pre, 1, 0, dp, P, PE, tile, p64::TILE_BYTES, d_rho, m, d_map, slot,
+    k_trsm64<<<dim3(nt, 1), TRSM_THREADS, TRSM_SMEM>>>(fronts, d_pre, 1, 0, dp, P, PE, tile, p64::TILE_BYTES, d_rho, m, d_map, slot,
                                              notpd, err, tcg::DEFAULT_WAIT);
   b.e = cudaGetLastError();
   if (b.e == cudaSuccess) b.e = cudaMemcpy(panel, P, PE * sizeof(double), cudaMemcpyDeviceToHost);

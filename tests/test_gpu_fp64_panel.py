@@ -137,3 +137,29 @@ def test_ill_conditioned_positive_definite_panels_are_not_flagged(panel, kappa):
         K *= 10.0 ** rng.uniform(-8, 8)
         P, D, bad = panel(np.concatenate([np.tril(K[:64, :64]), K[64:, :64]]), np.diag(K))
         assert bad is None
+
+
+@pytest.mark.parametrize("bw,rows", [(64, 200), (64, 1), (17, 130)])
+@pytest.mark.parametrize("noise", [1.0, 1e-2, 1e-4, 1e-8, 1e-12])
+def test_rows_below_are_solved_backward_stably(panel, noise, bw, rows):
+    """|B - X L^T| and |A - L L^T| within 4 units of 2^-53 of the products' scales whatever the tile's condition: X and L are
+    rounded to 2^-53 each (2 units together, by Cauchy-Schwarz), the digits and the residual's integers to 2^-55 and less.
+    Rows that are weakly correlated with the tile's columns keep to their own scale where its inverse is below 2^12."""
+    rng = np.random.default_rng(bw + rows)
+    n = bw + rows
+    x = np.sort(rng.uniform(0, 1, n))
+    K = np.exp(-0.5 * ((x[:, None] - x[None]) / 0.3) ** 2) + noise * np.eye(n)
+    B = K[bw:, :bw].copy()
+    weak = rng.uniform(size=rows) < 0.3
+    B[weak] *= 2.0 ** -30
+    P, D, bad = panel(np.concatenate([np.tril(K[:bw, :bw]), B]), np.diag(K))
+    assert bad is None
+    L, X = P[:bw].astype(np.longdouble), P[bw:].astype(np.longdouble)
+    d = np.sqrt(np.diag(K))
+    T = np.abs(np.tril(K[:bw, :bw] - L @ L.T)) / np.outer(d[:bw], d[:bw])
+    assert T.max() <= 4 * EPS, float(T.max() / EPS)
+    R = np.abs(B - X @ L.T) / d[None, :bw]
+    assert (R <= 4 * EPS * d[bw:, None]).all(), float(R.max() / EPS)
+    if noise >= 1e-4:
+        size = np.sqrt((X * X).sum(1, keepdims=True))
+        assert (R <= 4 * EPS * size).all(), float((R / size).max() / EPS)
