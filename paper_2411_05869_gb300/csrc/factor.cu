@@ -94,10 +94,8 @@ __global__ void __launch_bounds__(256) k_row_scale(DevPlan dp, int64_t n, const 
   rho[(int64_t)b * n + j] = ((e + 2) >> 1) - 1;
 }
 
-// The tensor-core operands of one level's large fronts: per front the six digit planes (m rows x ldk FP16, K contiguous)
-// of the columns of its current group, at ops + dp.op64_off.
 constexpr int KB = f64d::KG / T;   // blocks per group
-__device__ __forceinline__ int ldk_of(int w) { return T * min(KB, (w + T - 1) / T); }
+static_assert(KB == GP_GROUP64 && f64d::NS == GP_DIGITS64 && p64::TILE_BYTES == GP_TILE_BYTES64, "the plan's layout");
 
 // The updates F[i, j] -= sum_{l in K} L[i, l] L[j, l] on 128 x 64 tiles, j <= i, from the digit planes:
 //   LEFT: the columns of block kb (rows >= c0), K = the group's earlier blocks, before the block's POTRF;
@@ -414,17 +412,19 @@ static void factor_body(gp_ctx* ctx, gp_factor_t* f) {
   cudaStream_t st = ctx->stream;
   set_attrs();
   const int B = f->B;
-  const int64_t PE = sp.panel_entries, UE = sp.update_entries, IE = itile_bytes(sp);
+  const int64_t PE = sp.panel_entries, UE = sp.update64_entries, IE = UE * (int64_t)sizeof(double);
+  int32_t* rho = reinterpret_cast<int32_t*>(f->work);   // the scale exponent of every row of L, B x n (the solves come later)
   values_run(ctx, f);   // A3, A4 (zeroes and fills the panels)
   k_fill_i32<<<grid_for(B, 128), 128, 0, st>>>(f->notpd, B, INT_MAX);
   GP_CHECK_LAUNCH(ctx);
   GP_CUDA(cudaMemsetAsync(f->tiles_err, 0, sizeof(int32_t), st));
-  k_row_scale<<<dim3(grid_for(ps->n, 256), B), 256, 0, st>>>(dp, ps->n, f->panels, PE, f->rho);
+  k_row_scale<<<dim3(grid_for(ps->n, 256), B), 256, 0, st>>>(dp, ps->n, f->panels, PE, rho);
   GP_CHECK_LAUNCH(ctx);
   ProfLevelScope pls_(ctx);
   for (int32_t L = 0; L < sp.nlevels; L++) {
     const SymPlan::Level& lv = sp.levels[L];
     ctx->prof_level = L;
+    uint8_t* itile = reinterpret_cast<uint8_t*>(f->upd + lv.tile64_off);   // the step's tiles
     if (lv.asm_n > 0) {
       ProfScope ps_(ctx, KC_EXTEND_ADD);
       ea::k_assemble64<<<dim3((unsigned)lv.asm_n, B), ea::THREADS, 0, st>>>(dp.asm_tab + lv.asm_off, dp, f->panels,
@@ -449,7 +449,7 @@ static void factor_body(gp_ctx* ctx, gp_factor_t* f) {
       ProfScope ps_(ctx, group ? KC_UPDATE : KC_UPDATE_LEFT, B * u.flops);
       auto k = group ? k_update64<true> : k_update64<false>;
       k<<<grid, U64_THREADS, U64_SMEM, st>>>(dp.upd64_fronts + u.off, dp.upd64_pre + u.pre_off, u.n, u.total, ntiles,
-                                             kb, dp, f->op_maps, f->op_slot, f->rho, ps->n, f->panels, f->upd, PE, UE,
+                                             kb, dp, f->op_maps, f->op_slot, rho, ps->n, f->panels, f->upd, PE, UE,
                                              f->tiles_err, f->wait_lim);
       GP_CHECK_LAUNCH(ctx);
     };
@@ -459,22 +459,20 @@ static void factor_body(gp_ctx* ctx, gp_factor_t* f) {
       {
         ProfScope ps_(ctx, KC_POTRF, B * stp.potrf_flops);
         k_potrf64<<<dim3(2 * stp.nfront, B), p64::THREADS, sizeof(p64::Smem), st>>>(
-            fronts, stp.kb, dp, f->panels, PE, f->notpd, f->dinv, sp.diag_entries, f->itile, IE, f->tiles_err);
+            fronts, stp.kb, dp, f->panels, PE, f->notpd, f->dinv, sp.diag_entries, itile, IE, f->tiles_err);
         GP_CHECK_LAUNCH(ctx);
       }
       if (stp.trsm128_total > 0) {
         ProfScope ps_(ctx, KC_TRSM, B * stp.trsm_flops);
         k_trsm64<<<dim3((unsigned)stp.trsm128_total, B), TRSM_THREADS, TRSM_SMEM, st>>>(
-            fronts, dp.step_pre + stp.pre_off + stp.nfront + 1, stp.nfront, stp.kb, dp, f->panels, PE, f->itile, IE,
-            f->rho, ps->n, f->op_maps, f->op_slot, f->notpd, f->tiles_err, f->wait_lim);
+            fronts, dp.step_pre + stp.pre_off + stp.nfront + 1, stp.nfront, stp.kb, dp, f->panels, PE, itile, IE,
+            rho, ps->n, f->op_maps, f->op_slot, f->notpd, f->tiles_err, f->wait_lim);
         GP_CHECK_LAUNCH(ctx);
       }
       if (stp.group64.total > 0) update(stp.group64, stp.kb, true);
     }
   }
 }
-
-int64_t itile_bytes(const SymPlan& sp) { return sp.max_large * (int64_t)p64::TILE_BYTES; }
 
 // The tensor maps of the FP64 path's digit planes, one per large front: 4-D (columns of a group x rows x digit planes x
 // proposals), boxes of 64 columns x 64 rows with the 128-byte swizzle; rows past the front read as zeros.
@@ -493,9 +491,9 @@ void build_digit_maps(gp_ctx* ctx, gp_factor_t* f) {
     const int32_t s = order[k];
     const int64_t m = (int64_t)sp.sn_w[s] + sp.sn_r[s], ldk = sp.op64_ldk(s);
     cuuint64_t dims[4] = {(cuuint64_t)ldk, (cuuint64_t)m, (cuuint64_t)f64d::NS, (cuuint64_t)f->B};
-    cuuint64_t strides[3] = {(cuuint64_t)ldk * 2, (cuuint64_t)(m * ldk) * 2, (cuuint64_t)sp.op64_entries * 2};
+    cuuint64_t strides[3] = {(cuuint64_t)ldk * 2, (cuuint64_t)(m * ldk) * 2, (cuuint64_t)sp.update64_entries * 8};
     cuuint32_t box[4] = {T, T, 1, 1}, es[4] = {1, 1, 1, 1};
-    CUresult r = enc(&maps[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, f->op64 + sp.sn_op64_off[s], dims, strides, box, es,
+    CUresult r = enc(&maps[k], CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, f->upd + sp.sn_op64_off[s], dims, strides, box, es,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     GP_REQUIRE(r == CUDA_SUCCESS, "cuTensorMapEncodeTiled rejected a digit map");

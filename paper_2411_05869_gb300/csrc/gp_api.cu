@@ -377,7 +377,6 @@ gp_status assemble_common(gp_ctx* ctx, const double* d_X, int64_t n, int d, cons
     dp.loff32 = upload(ctx, ps->bufs, sp.sn_loff32);
     dp.lo_off = upload(ctx, ps->bufs, sp.sn_lo_off);
     dp.doff = upload(ctx, ps->bufs, sp.sn_doff);
-    dp.op64_off = upload(ctx, ps->bufs, sp.sn_op64_off);
     dp.upd64_fronts = upload(ctx, ps->bufs, sp.upd64_fronts);
     dp.upd64_pre = upload(ctx, ps->bufs, sp.upd64_pre);
     dp.large_kb = upload(ctx, ps->bufs, sp.large_kb);
@@ -586,10 +585,7 @@ extern "C" gp_status gp_factor_core(gp_ctx* ctx, gp_pointset* ps, const gp_hyper
     if (f->core_kind == GP_CORE_PACIOREK) f->Cpt = dalloc<double>(ctx, f->bufs, (size_t)B * ps->n * 2);
     if (prec == GP_FP64) {
       f->panels = dalloc<double>(ctx, f->bufs, (size_t)B * sp.panel_entries);
-      f->upd = dalloc<double>(ctx, f->bufs, (size_t)B * sp.update_entries);
-      f->op64 = dalloc<__half>(ctx, f->bufs, (size_t)B * sp.op64_entries);
-      f->itile = dalloc<uint8_t>(ctx, f->bufs, (size_t)B * itile_bytes(sp));
-      f->rho = dalloc<int32_t>(ctx, f->bufs, (size_t)B * ps->n);
+      f->upd = dalloc<double>(ctx, f->bufs, (size_t)B * sp.update64_entries);
       build_digit_maps(ctx, f);
     } else {
       if (!ps->dest32) {   // the point set's own context owns (and stream-orders) its per-precision map
@@ -658,8 +654,7 @@ size_t factor_bytes(const gp_pointset* ps, gp_precision prec, int B, const Theta
     }
   nmaps = std::max<size_t>(nmaps, 1);
   if (prec == GP_FP64) {
-    t += alloc_bytes(b * sp.panel_entries * 8) + alloc_bytes(b * sp.update_entries * 8) +
-         alloc_bytes(b * sp.op64_entries * 2) + alloc_bytes(b * itile_bytes(sp)) + alloc_bytes(b * n * 4) + alloc_bytes(nmaps * 128) +
+    t += alloc_bytes(b * sp.panel_entries * 8) + alloc_bytes(b * sp.update64_entries * 8) + alloc_bytes(nmaps * 128) +
          alloc_bytes((sp.sn_w.size() + 1) * 4);
   } else {
     t += alloc_bytes(b * sp.panel32_entries * 4) + alloc_bytes(b * sp.diag_entries * 8) +

@@ -16,7 +16,6 @@
 
 #include <cuda.h>
 #include <cudaTypedefs.h>
-#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 #include <stdint.h>
 
@@ -167,6 +166,8 @@ void d2h(gp_ctx* ctx, T* dst, const T* src, size_t count) {
 // Host-side result of A6, plus the device copies the numeric kernels read.
 #define GP_GROUP 8   // default 64-column blocks per deferred-update group of the mixed path
 #define GP_GROUP64 4 // 64-column blocks per deferred-update group of the FP64 path (K = 256: f64_digits.cuh)
+#define GP_DIGITS64 6         // digit planes of the FP64 path's operands (f64_digits.cuh)
+#define GP_TILE_BYTES64 98816 // a diagonal tile and its inverse as digit planes, and their exponents (potrf64.cuh)
 #define GP_TN_LEFT 64     // tensor-core tile width (columns) of the mixed path's left-looking block updates
 #define GP_TN_GROUP 256   // default tile width of its group-end updates (rows stay 128 per tile)
 
@@ -212,12 +213,12 @@ struct SymPlan {
   std::vector<int32_t> upd_fronts;   // per step: fronts of the left-looking and of the group update
   std::vector<int64_t> upd_pre;      // their tile prefixes
 
-  // FP64 path: the digit planes of a level's large fronts (f64_digits.cuh), per front 6 planes of m rows x op64_ldk
-  // FP16 (the columns of its current group of GP_GROUP64 blocks), at sn_op64_off in a workspace of op64_entries FP16
-  // that every level and every group reuse
+  // FP64 path: the digit planes of a level's large fronts (f64_digits.cuh), per front GP_DIGITS64 planes of m rows x
+  // op64_ldk FP16 (the columns of its current group of GP_GROUP64 blocks), and the tiles of its current step
+  // (GP_TILE_BYTES64 per large front of the level) lie in the update workspace, where the level's children have left
+  // room after its assembly, and past its end where that is not enough. Offsets in entries, multiples of 16.
   std::vector<int64_t> sn_op64_off;
-  int64_t op64_entries = 64;
-  int64_t max_large = 1;   // most large fronts of a level (the FP64 path's inverse tiles of one step)
+  int64_t update64_entries = 16;   // the FP64 path's update workspace: update_entries or more, a multiple of 16
   int64_t op64_ldk(int64_t s) const {
     return GP_TILE * std::min<int64_t>(GP_GROUP64, (sn_w[s] + GP_TILE - 1) / GP_TILE);
   }
@@ -244,6 +245,7 @@ struct SymPlan {
                       Upd64 left64, group64;   // the same updates of the FP64 path (128 x 64 tiles)
                       double potrf_flops, trsm_flops; };   // useful flops of the step's launches
   struct Level {
+    int64_t tile64_off = 0;          // FP64 path: the tiles of the level's steps in the update workspace
     int64_t asm_off = 0, asm_n = 0;  // into asm_tab: the assembly's runs of rows
     int64_t small_off = 0; int32_t nsmall = 0;   // into small_list
     std::vector<StepLaunch> steps;   // large fronts, one per block column
@@ -290,7 +292,6 @@ struct DevPlan {
   int32_t* ldw;
   int64_t *loff32, *doff;
   int64_t* lo_off;
-  int64_t* op64_off;
   int32_t* upd64_fronts;
   int64_t* upd64_pre;
   int32_t* large_kb;
@@ -385,10 +386,7 @@ struct gp_factor_s {
   unsigned long long refine_runs_seen = 0;     // corrections already added to the context's launch count
   int32_t* tiles_err = nullptr; // set when a bounded wait (tensor-core updates, solve tasks) ran out
   int32_t* flow_sync = nullptr; // the solve tasks' tickets and readiness flags (flow_sync_entries)
-  __half* op64 = nullptr;       // GP_FP64: the digit planes of one level's large fronts, B x op64_entries
-  uint8_t* itile = nullptr;     // GP_FP64: the inverse tiles of one step as digit planes, B x max_large x 49,664 bytes
-  int32_t* rho = nullptr;       // GP_FP64: the scale exponent of every row of L, B x n
-  double* upd = nullptr;        // B x update_entries
+  double* upd = nullptr;        // GP_FP64: B x update64_entries
   float* upd32 = nullptr;
   double* val = nullptr;        // B x nnz CSR values of C_z (refinement SpMV)
   int32_t* notpd = nullptr;     // B: smallest failing permuted column (INT_MAX = none)
@@ -451,7 +449,6 @@ void compute_dest_map(gp_ctx* ctx, gp_pointset* ps);
 void compute_dest_map_mixed(gp_ctx* ctx, gp_pointset* ps);
 void build_update_maps(gp_ctx* ctx, gp_factor_t* f);
 void build_digit_maps(gp_ctx* ctx, gp_factor_t* f);
-int64_t itile_bytes(const SymPlan& sp);   // of one proposal
 PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder();
 int64_t bwd_part_entries(const SymPlan& sp);
 // The solve tasks' tickets (forward and backward, one each per level) and readiness flags (forward and

@@ -379,6 +379,9 @@ void build_symbolic(int64_t n, const int64_t* rowptr, const int32_t* col, const 
   sp.sn_uoff.assign(ns, 0);
   {
     FirstFit ff;
+    sp.sn_op64_off.assign(ns, 0);
+    sp.levels.assign(sp.nlevels, SymPlan::Level());
+    int64_t end64 = 1;
     for (int32_t L = 0; L < sp.nlevels; L++) {
       for (int32_t q = sp.lev_ptr[L]; q < sp.lev_ptr[L + 1]; q++) {
         int32_t s = sp.lev_sn[q];
@@ -392,16 +395,26 @@ void build_symbolic(int64_t n, const int64_t* rowptr, const int32_t* col, const 
           ff.release(sp.sn_uoff[ch], (int64_t)sp.sn_r[ch] * sp.sn_r[ch]);
         }
       }
+      // the FP64 path's digit planes and tiles of this level: among what is free now, for this level alone
+      FirstFit level = ff;
+      auto aligned = [&](int64_t bytes) { return (level.alloc((bytes + 7) / 8 + 15) + 15) / 16 * 16; };
+      int64_t nlarge = 0;
+      for (int32_t q = sp.lev_ptr[L]; q < sp.lev_ptr[L + 1]; q++) {
+        const int32_t s = sp.lev_sn[q];
+        const int64_t m = (int64_t)sp.sn_w[s] + sp.sn_r[s];
+        if (m <= GP_SMALL_M) continue;
+        nlarge++;
+        sp.sn_op64_off[s] = aligned(GP_DIGITS64 * m * sp.op64_ldk(s) * 2);
+      }
+      if (nlarge > 0) sp.levels[L].tile64_off = aligned(nlarge * GP_TILE_BYTES64);
+      end64 = std::max(end64, level.peak);
     }
     sp.update_entries = std::max<int64_t>(ff.peak, 1);
+    sp.update64_entries = (std::max(sp.update_entries, end64) + 15) / 16 * 16;
   }
 
   // ---- launch schedule
-  sp.levels.assign(sp.nlevels, SymPlan::Level());
   sp.sn_lo_off.assign(sp.ns, 0);
-  sp.sn_op64_off.assign(sp.ns, 0);
-  sp.op64_entries = 64;
-  sp.max_large = 1;
   sp.lo_entries = 8;
   sp.level_large.assign(sp.nlevels, SymPlan::LevelLarge());
   sp.sn_fl.assign(sp.ns, -1);
@@ -552,13 +565,6 @@ void build_symbolic(int64_t n, const int64_t* rowptr, const int32_t* col, const 
         lo += (int64_t)(sp.sn_w[s] + sp.sn_r[s]) * ((sp.sn_ldw[s] + 7) / 8 * 8);
       }
       sp.lo_entries = std::max(sp.lo_entries, lo);
-      int64_t o64 = 0;   // the FP64 path's digit planes: rows of op64_ldk FP16 (a multiple of 128 bytes)
-      for (int32_t s : large) {
-        sp.sn_op64_off[s] = o64;
-        o64 += 6 * (int64_t)(sp.sn_w[s] + sp.sn_r[s]) * sp.op64_ldk(s);
-      }
-      sp.op64_entries = std::max(sp.op64_entries, o64);
-      sp.max_large = std::max<int64_t>(sp.max_large, (int64_t)large.size());
     }
     // dataflow solve tasks of this level's large fronts (SB blocks of 64 columns per chain task: 2 where the
     // level's chains are long, else 1; rows below the columns in tasks of 64 SB rows): forward tasks ordered by

@@ -218,3 +218,18 @@ def test_log_likelihoods_are_as_accurate_as_an_fp64_cholesky(n, noise):
         ps.free()
     rms = lambda v: math.sqrt(np.mean(np.square(v)))
     assert rms(got) <= 16 * rms(host), (rms(got), rms(host))
+
+
+def test_digit_planes_take_no_memory_of_their_own_beside_update_matrices():
+    """The operands of a level lie where its children's update matrices were: the factor of this plan takes 114,011,904
+    bytes without them (panels, update matrices, inverses, values and the solves' vectors), and at most 1 % more with."""
+    from paper_2411_05869_gb300 import gp
+    w = synth.uniform_spacetime(9000, 0, 60.0, 16, 1, ndays=66)
+    ctx = gp.Context(0)
+    ps = ctx.assemble(_dev(w.X), w.hyper.core_radius)
+    need = ps.factor_bytes(w.hyper, 1, gp.GP_FP64)
+    assert need <= 1.01 * 114011904
+    f = ctx.factor(ps, [w.hyper], gp.GP_FP64)
+    assert f.info()["bytes"] == need
+    f.free()
+    ps.free()
