@@ -1,16 +1,23 @@
-// f64_digits.cuh -- FP64 products on the FP16 tensor cores: an FP64 entry as six signed 9-bit digits.
+// f64_digits.cuh -- FP64 products on the FP16 tensor cores: an FP64 entry as six signed 9-bit digits (the error-free
+// splitting of matrix products of Ozaki, Ogita, Oishi and Rump, on fixed-point rows).
 //
 // GB300's FP64 pipe runs at about 1 TFLOP/s (0.5 lanes per clock and scheduler), its FP16 tensor cores at 1.7
 // PFLOP/s. An entry x with |x| <= 2^(rho + 1) is the fixed-point number x = 2^rho sum_{s < 6} d_s 2^(-9 (s + 1)) + e
 // with |d_0| <= 1024, |d_s| <= 256 for s > 0 and |e| <= 2^(rho - 55): every digit is exact in FP16, every product of
 // two digits exact in FP32, and a dot product's sum over one level l = s + t, A_l = sum_k sum_{s + t = l} d_s d'_t, is
-// an integer, which the FP32 accumulator holds exactly below 2^24. For two rows of a Cholesky factor with 2^(rho + 1)
-// >= sqrt(C_ii), the rows' squared norms are at most C_ii, so over K = 256 level 0 is below 2^21 and level 1 below 2^23
-// (Cauchy-Schwarz); the lower levels' digits are noise-like, and even the sum of 256 squares of them is at most 2^24.
-// Two general operands take |x| <= 2^rho (|d_0| <= 512) and K = 64. The 26 digit products of the levels 0..6 are kept;
-// the dropped ones (l >= 7) and the remainders e leave a relative error of about 2^-58 sqrt(C_ii C_jj), below the
-// rounding of a chain of K FP64 multiply-adds (2^-53 of the running sum per step). The levels are put together in 64-bit
-// integers and rounded to FP64 once.
+// an integer, which the FP32 accumulator holds exactly up to 2^24. For two rows of a Cholesky factor with 2^(rho + 1)
+// >= sqrt(C_ii), the rows' squared norms are at most C_ii, so over K = 256 level 0 is at most 2^20 and level 1 2^23
+// (Cauchy-Schwarz). The lower levels have no such bound: level l adds up l + 1 digit products, each at most 2^24 (2^22 with
+// digit 0). Their digits are noise-like, so that only squares of the same digits add up: on covariances of uniform points,
+// lattices, duplicates and points of common bumps the largest sums measured 0.5 times 2^24, 0.99 at the most (32 bump
+// families of points without any other covariance). More would take some 150 columns of a group with entries equal to 2^-18 of
+// the scale in two rows, that is, columns without covariance among themselves and with the same covariance to both rows:
+// an arrow matrix of 256 such columns reached 2.5 times 2^24, at level 6. A sum beyond 2^24 is rounded to even numbers, to a
+// unit of its level, 2^(-18 - 9 l) of the scales: 2^-45 at level 3, less than FP64's rounding from level 4 on.
+// The 26 digit products of the levels 0..6 are kept; the dropped ones (l >= 7) and the remainders e leave an error of about
+// 2^-58 sqrt(C_ii C_jj), below the rounding of a chain of K FP64 multiply-adds of rows of that length (2^-53 of the running
+// sum per step); a row's entries far below its scale keep fewer than 53 bits. The levels are put together in 64-bit integers
+// and rounded to FP64 once.
 #pragma once
 #include <cuda_fp16.h>
 #include <stdint.h>
@@ -20,13 +27,6 @@ namespace f64d {
 constexpr int NS = 6;     // digits of an entry
 constexpr int NL = 7;     // levels s + t kept
 constexpr int KG = 256;   // columns of a deferred-update group: the longest sum of one accumulation
-
-// The smallest rho with |x| <= 2^rho from the exponent field (a NaN or an infinity gives some value: its factorization
-// is reported as not positive definite).
-__device__ __forceinline__ int rho_of(double x) {
-  const int e = (__double2hiint(x) >> 20) & 0x7ff;
-  return e == 0 ? -1022 : e - 1022;   // |x| < 2^(e - 1022)
-}
 
 // A fixed-point entry is kept in units of 2^-61 of its scale 2^rho, seven bits below the last digit. Digit s > 0 plus
 // 256 is the 9-bit field at bit 7 + 9 (5 - s) of the entry plus BIAS (256 in every field, and half a digit unit, so that
@@ -115,11 +115,6 @@ __device__ __forceinline__ double to_double(const Norm& r) {
   hi = zero ? 0u : hi | ((uint32_t)r.sg & 0x80000000u);
   lo = zero ? 0u : lo;
   return __hiloint2double((int)hi, (int)lo);
-}
-// The same number as a biased fixed-point entry at scale 2^rho.
-__device__ __forceinline__ int64_t to_biased(const Norm& r, int rho) {
-  const int n = min(max(rho + 1 - r.e, 0), 63);
-  return ((int64_t)(r.n >> n) ^ (int64_t)r.sg) + BIAS;
 }
 __device__ __forceinline__ double fix2double(int64_t v, int e) { return to_double(normalise(v, e + 62)); }   // v 2^e
 

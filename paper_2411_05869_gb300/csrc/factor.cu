@@ -97,6 +97,33 @@ __global__ void __launch_bounds__(256) k_row_scale(DevPlan dp, int64_t n, const 
 constexpr int KB = f64d::KG / T;   // blocks per group
 static_assert(KB == GP_GROUP64 && f64d::NS == GP_DIGITS64 && p64::TILE_BYTES == GP_TILE_BYTES64, "the plan's layout");
 
+// Eight consecutive columns of the seven level accumulators (ld columns apart) of this thread's lane.
+__device__ __forceinline__ void tmem_ld_levels(uint32_t ta, int ld, float (&a)[f64d::NL][8]) {
+  uint32_t r[f64d::NL * 8];
+  static_assert(f64d::NL == 7, "the wait below takes seven levels");
+#pragma unroll
+  for (int l = 0; l < f64d::NL; l++)
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
+                 : "=r"(r[8 * l]), "=r"(r[8 * l + 1]), "=r"(r[8 * l + 2]), "=r"(r[8 * l + 3]), "=r"(r[8 * l + 4]),
+                   "=r"(r[8 * l + 5]), "=r"(r[8 * l + 6]), "=r"(r[8 * l + 7])
+                 : "r"(ta + l * ld));
+  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                 "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                 "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
+                 "+r"(r[29]), "+r"(r[30]), "+r"(r[31]), "+r"(r[32]), "+r"(r[33]), "+r"(r[34]), "+r"(r[35]),
+                 "+r"(r[36]), "+r"(r[37]), "+r"(r[38]), "+r"(r[39]), "+r"(r[40]), "+r"(r[41]), "+r"(r[42]),
+                 "+r"(r[43]), "+r"(r[44]), "+r"(r[45]), "+r"(r[46]), "+r"(r[47]), "+r"(r[48]), "+r"(r[49]),
+                 "+r"(r[50]), "+r"(r[51]), "+r"(r[52]), "+r"(r[53]), "+r"(r[54]), "+r"(r[55])
+               :
+               : "memory");
+#pragma unroll
+  for (int l = 0; l < f64d::NL; l++)
+#pragma unroll
+    for (int c = 0; c < 8; c++) a[l][c] = __uint_as_float(r[8 * l + c]);
+}
+
 // The updates F[i, j] -= sum_{l in K} L[i, l] L[j, l] on 128 x 64 tiles, j <= i, from the digit planes:
 //   LEFT: the columns of block kb (rows >= c0), K = the group's earlier blocks, before the block's POTRF;
 //   GROUP: rows and columns after the group, tiles on and below the diagonal, K = the whole group.
@@ -105,11 +132,12 @@ static_assert(KB == GP_GROUP64 && f64d::NS == GP_DIGITS64 && p64::TILE_BYTES == 
 // it as it lands (26 products of 4 instructions per 64 columns of K, into one accumulator per level: 7 x 64 TMEM
 // columns), warps 2-9 put the levels together in 64-bit integers and subtract from the front in FP64 -- lanes are rows,
 // so the column-major front is read and written in whole 256-byte segments. The seven accumulators fill the tensor
-// memory, so a tile's epilogue does not overlap the next tile's MMAs (its operand loads do). 128 x 64 x 16
-// instructions read 6 KB of shared memory in the 32 clocks they multiply: about two thirds of the FP16 peak.
+// memory, so a tile's epilogue does not overlap the next tile's MMAs (its operand loads do): the tensor pipe is busy 60 % of
+// the time, and with N = 64 an instruction (6 KB of shared memory read in 48 clocks) uses half of its rate. A group end of 5744
+// rows: 326 us, tensor cycles 30 %, DRAM 9 % (counters of one launch), 0.35 of the measured FP16 rate in digit products.
 // Against FP64 multiply-adds (64-column updates of the whole trailing matrix at the FP64 pipe's 1 TFLOP/s) the updates
-// of one factorization went from 101.8 to 9.4 ms at n = 100k (1.1e11 flops) and from 725 to 42 ms at n = 200k (8.3e11
-// flops); residuals |r - C alpha| / |r| stayed the same.
+// of one factorization went from 101.8 to 10.3 ms at n = 100k (1.1e11 flops) and from 725 to 47 ms at n = 200k (8.3e11
+// flops), left-looking strips included; residuals |r - C alpha| / |r| stayed the same.
 constexpr int U64_THREADS = 320, U64_SLOTS = 9, U64_SLOT = (128 + T) * 128;
 constexpr int U64_SMEM = U64_SLOTS * U64_SLOT + 256 + 1024;
 

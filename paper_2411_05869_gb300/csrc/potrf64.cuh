@@ -2,7 +2,7 @@
 //
 // The tile is one link of the factorization's chain of dependent steps, so its latency counts. GB300's FP64 pipe takes
 // 64 clocks for each warp instruction of a scheduler (0.5 lanes per clock); the integer pipe's 32 x 32 + 64 multiply-add
-// takes 2. The elimination with its inverse in FP64 registers took 133 us per tile, this takes 42. Here both run in 60-bit fixed
+// takes 2. The elimination with its inverse in FP64 registers took 133 us per tile, this takes 44. Here both run in 60-bit fixed
 // point on the integer pipe, on a cluster of two CTAs: the first eliminates the tile a column at a time, the second forms
 // the inverse of the factor a column or two behind, from the columns that the first writes into its shared memory. (On
 // one CTA the two together keep the integer pipe busy for about 700 clocks per column; apart, each is bounded by its chain

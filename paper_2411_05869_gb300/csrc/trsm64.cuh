@@ -9,34 +9,8 @@
 
 namespace {
 
-// Eight consecutive columns of the seven level accumulators (ld columns apart) of this thread's lane.
-__device__ __forceinline__ void tmem_ld_levels(uint32_t ta, int ld, float (&a)[f64d::NL][8]) {
-  uint32_t r[f64d::NL * 8];
-  static_assert(f64d::NL == 7, "the wait below takes seven levels");
-#pragma unroll
-  for (int l = 0; l < f64d::NL; l++)
-    asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];\n"
-                 : "=r"(r[8 * l]), "=r"(r[8 * l + 1]), "=r"(r[8 * l + 2]), "=r"(r[8 * l + 3]), "=r"(r[8 * l + 4]),
-                   "=r"(r[8 * l + 5]), "=r"(r[8 * l + 6]), "=r"(r[8 * l + 7])
-                 : "r"(ta + l * ld));
-  asm volatile("tcgen05.wait::ld.sync.aligned;\n"
-               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
-                 "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
-                 "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
-                 "+r"(r[29]), "+r"(r[30]), "+r"(r[31]), "+r"(r[32]), "+r"(r[33]), "+r"(r[34]), "+r"(r[35]),
-                 "+r"(r[36]), "+r"(r[37]), "+r"(r[38]), "+r"(r[39]), "+r"(r[40]), "+r"(r[41]), "+r"(r[42]),
-                 "+r"(r[43]), "+r"(r[44]), "+r"(r[45]), "+r"(r[46]), "+r"(r[47]), "+r"(r[48]), "+r"(r[49]),
-                 "+r"(r[50]), "+r"(r[51]), "+r"(r[52]), "+r"(r[53]), "+r"(r[54]), "+r"(r[55])
-               :
-               : "memory");
-#pragma unroll
-  for (int l = 0; l < f64d::NL; l++)
-#pragma unroll
-    for (int c = 0; c < 8; c++) a[l][c] = __uint_as_float(r[8 * l + c]);
-}
-
-// Four columns of the levels 0..3, and of the levels 4..6 where `deep` (zero otherwise).
+// Four consecutive columns (this thread's lane) of the accumulators of the levels 0..3, ld columns apart, and of the levels
+// 4..6 where `deep` (zero otherwise).
 __device__ __forceinline__ void tmem_ld_levels4(uint32_t ta, int ld, bool deep, float (&a)[f64d::NL][4]) {
   uint32_t r[16], q[12];
 #pragma unroll
