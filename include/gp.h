@@ -52,7 +52,9 @@ typedef enum {
 } gp_status;
 
 typedef enum {
-  GP_FP64 = 0,         /* every step in FP64 */
+  GP_FP64 = 0,         /* every step in FP64, but for the factorization's products and diagonal tiles, whose backward
+                          errors are at or below FP64's on the rows' scales (FP64 entries as nine-bit digits on the
+                          tensor cores, 60-bit fixed point) */
   GP_MIXED = 1         /* off-diagonal supernode updates on tensor cores with FP32 accumulation, each FP32 operand
                           split into an FP16 pair (or a TF32 pair: GP_OPT_SPLIT_F16), and FP32 off-diagonal
                           storage; diagonal-block factorization, log-det and refinement residuals in FP64 (the

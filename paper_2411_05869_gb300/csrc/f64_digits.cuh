@@ -10,9 +10,9 @@
 // (Cauchy-Schwarz). The lower levels have no such bound: level l adds up l + 1 digit products, each at most 2^24 (2^22 with
 // digit 0). Their digits are noise-like, so that only squares of the same digits add up: on covariances of uniform points,
 // lattices, duplicates and points of common bumps the largest sums measured 0.5 times 2^24, 0.99 at the most (32 bump
-// families of points without any other covariance). More would take some 150 columns of a group with entries equal to 2^-18 of
-// the scale in two rows, that is, columns without covariance among themselves and with the same covariance to both rows:
-// an arrow matrix of 256 such columns reached 2.5 times 2^24, at level 6. A sum beyond 2^24 is rounded to even numbers, to a
+// families of points without any other covariance). More takes some 150 columns of a group with entries equal to 2^-18 of
+// the scale in two rows, that is, columns with the same covariance to both rows and nearly none among themselves (replicates
+// at the foot of one bump, without a core term): an arrow matrix of 256 such columns reached 2.5 times 2^24, at level 6. A sum beyond 2^24 is rounded to even numbers, to a
 // unit of its level, 2^(-18 - 9 l) of the scales: 2^-45 at level 3, less than FP64's rounding from level 4 on.
 // The 26 digit products of the levels 0..6 are kept; the dropped ones (l >= 7) and the remainders e leave an error of about
 // 2^-58 sqrt(C_ii C_jj), below the rounding of a chain of K FP64 multiply-adds of rows of that length (2^-53 of the running
